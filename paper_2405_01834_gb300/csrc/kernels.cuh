@@ -68,6 +68,8 @@ struct QuartetLaunch {
   const double* const* mol_D;
   double* const* mol_K;
   const int32_t* mol_nao;
+  // register kernel: 2^(split_b + split_k) lanes share a quartet's primitives (set by its launcher)
+  int32_t split_b, split_k;
   // solid-harmonic launches (plan.sph): global staging, xg_doubles per team of the launch grid
   double* sph_scratch;
 };

@@ -13,6 +13,7 @@
 // gradient launches use the team kernel.
 #pragma once
 
+#include <algorithm>
 #include <utility>
 
 #include "kernels.cuh"
@@ -101,8 +102,15 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
   constexpr int EB = etab_size(LA, LB), EK = etab_size(LC, LD);
 
   extern __shared__ double xs_smem[];
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= a.nq) return;
+  // 2^(split_b + split_k) neighbouring lanes share a quartet: lane (sb, sk) takes the bra primitive pairs
+  // sb, sb + Sb, ... and of each the ket primitive pairs sk, sk + Sk, ... (see split_of)
+  const int lS = a.split_b + a.split_k, S = 1 << lS;
+  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t q = gid >> lS;
+  if (q >= a.nq) return;   // whole lane groups leave together
+  const int sub = (int)gid & (S - 1);
+  const int Sb = 1 << a.split_b, Sk = 1 << a.split_k, sb = sub >> a.split_k, sk = sub & (Sk - 1);
+  const unsigned grp = (S == 32 ? 0xffffffffu : (1u << S) - 1u) << (threadIdx.x & 31 & ~(S - 1));
   const int2 qp = a.qpairs[q];
   const double* __restrict__ rb0 = a.recs + a.pair_rec[qp.x + a.bra_var_off];
   const double* __restrict__ rk0 = a.recs_signed + a.pair_rec[qp.y + a.ket_var_off];
@@ -116,13 +124,15 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
   TArr<XS, Nb * Nk> V;
   TArr<XS, HB * Nk> X;
   if constexpr (XS) {
-    V.p = xs_smem + threadIdx.x;
+    V.p = xs_smem + (threadIdx.x & ~(S - 1));   // the shellset column of the group's first lane
     X.p = xs_smem + (VSH ? Nb * Nk : 0) * kXsBlock + threadIdx.x;
   }
-  if constexpr (!XS || VSH) sfor<Nb * Nk>([&](auto i) { V[i] = 0.0; });
+  if constexpr (!XS) sfor<Nb * Nk>([&](auto i) { V[i] = 0.0; });
   double* const outq = DIGEST ? nullptr : a.out + (a.qout ? a.qout[q] : q * (int64_t)(Nb * Nk));
 
-  for (int pb = 0; pb < Kb; ++pb) {
+  for (int pb0 = 0; pb0 < Kb; pb0 += Sb) {
+    const bool live = pb0 + sb < Kb;   // a lane past the last bra primitive adds zeros to the group's sums
+    const int pb = live ? pb0 + sb : 0;
     const double* __restrict__ rb = rb0 + (int64_t)pb * RB;
     const double zp = __ldg(rb), izp = __ldg(rb + 1);
     const double Px = __ldg(rb + 2), Py = __ldg(rb + 3), Pz = __ldg(rb + 4);
@@ -130,7 +140,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
     const double prefb = 34.986836655249725693 * izp * __ldg(rb + 5);
     sfor<HB * Nk>([&](auto i) { X[i] = 0.0; });
 
-    for (int pk = 0; pk < Kk; ++pk) {
+    for (int pk = live ? sk : Kk; pk < Kk; pk += Sk) {
       const double* __restrict__ rk = rk0 + (int64_t)pk * RK;
       const double zq = __ldg(rk), izq = __ldg(rk + 1);
       const double PQx = Px - __ldg(rk + 2), PQy = Py - __ldg(rk + 3), PQz = Pz - __ldg(rk + 4);
@@ -261,13 +271,26 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
             }
           }
           const int o = (ia * NB + ib) * Nk;
-          if constexpr (VSH) {
-            sfor<Nk>([&](auto cd) { V[o + cd] += acc[cd]; });
-          } else if (pb == 0) {
-            sfor<Nk>([&](auto cd) { outq[o + cd] = acc[cd]; });
-          } else {
-            sfor<Nk>([&](auto cd) { outq[o + cd] += acc[cd]; });
+          if (S == 1) {
+            if constexpr (VSH) {
+              if (pb0 == 0) sfor<Nk>([&](auto cd) { V[o + cd] = acc[cd]; });
+              else sfor<Nk>([&](auto cd) { V[o + cd] += acc[cd]; });
+            } else if (pb0 == 0) {
+              sfor<Nk>([&](auto cd) { outq[o + cd] = acc[cd]; });
+            } else {
+              sfor<Nk>([&](auto cd) { outq[o + cd] += acc[cd]; });
+            }
+            continue;
           }
+          for (int off = 1; off < S; off <<= 1)   // the group's sum, in every lane
+            sfor<Nk>([&](auto cd) { acc[cd] += __shfl_xor_sync(grp, acc[cd], off); });
+          sfor<Nk>([&](auto cd) {
+            if ((cd & (S - 1)) != sub) return;   // the lanes of the group share the row's elements
+            double* dst;
+            if constexpr (VSH) dst = &V[o + cd];
+            else dst = outq + o + cd;
+            *dst = pb0 == 0 ? acc[cd] : *dst + acc[cd];
+          });
         }
       }
     } else {
@@ -302,9 +325,20 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
     }
   }
 
+  if constexpr (!XS) {
+    for (int off = 1; off < S; off <<= 1)
+      sfor<Nb * Nk>([&](auto i) { V[i] += __shfl_xor_sync(grp, V[i], off); });
+  }
+  if constexpr (VSH) __syncwarp(grp);   // every lane reads the shellset below
   if constexpr (!DIGEST) {
     // (no offsets: shellsets back to back); the shared-memory variant has written its rows already
-    if constexpr (!XS) sfor<Nb * Nk>([&](auto i) { outq[i] = V[i]; });
+    if constexpr (!XS) {
+      if (S == 1) sfor<Nb * Nk>([&](auto i) { outq[i] = V[i]; });
+      else
+        sfor<Nb * Nk>([&](auto i) {
+          if ((i & (S - 1)) == sub) outq[i] = V[i];
+        });
+    }
   } else {
     // Exchange digestion of the unique quartet (ij|kl) with weight w, as in
     // the team kernel: K_ik += w D_jl V, K_il += w D_jk V, K_jk += w D_il V,
@@ -322,12 +356,14 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
       auto Vr = [&](int x, int b, int c, int d) -> double { return V[((x * NB + b) * NC + c) * ND + d]; };
       for (int x = 0; x < NA; ++x) {
         for (int c = 0; c < NC; ++c) {   // K_ik
+          if (((x * NC + c) & (S - 1)) != sub) continue;   // the group's lanes share the elements of each block
           double s1 = 0.0;
           for (int b = 0; b < NB; ++b)
             for (int d = 0; d < ND; ++d) s1 = fma(__ldg(D + (aj + b) * nao + al + d), Vr(x, b, c, d), s1);
           atomicAdd(K + (ai + x) * nao + ak + c, w * s1);
         }
         for (int d = 0; d < ND; ++d) {   // K_il
+          if (((x * ND + d) & (S - 1)) != sub) continue;
           double s2 = 0.0;
           for (int b = 0; b < NB; ++b)
             for (int c = 0; c < NC; ++c) s2 = fma(__ldg(D + (aj + b) * nao + ak + c), Vr(x, b, c, d), s2);
@@ -336,12 +372,14 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
       }
       for (int x = 0; x < NB; ++x) {
         for (int c = 0; c < NC; ++c) {   // K_jk
+          if (((x * NC + c) & (S - 1)) != sub) continue;
           double s3 = 0.0;
           for (int y = 0; y < NA; ++y)
             for (int d = 0; d < ND; ++d) s3 = fma(__ldg(D + (ai + y) * nao + al + d), Vr(y, x, c, d), s3);
           atomicAdd(K + (aj + x) * nao + ak + c, w * s3);
         }
         for (int d = 0; d < ND; ++d) {   // K_jl
+          if (((x * ND + d) & (S - 1)) != sub) continue;
           double s4 = 0.0;
           for (int y = 0; y < NA; ++y)
             for (int c = 0; c < NC; ++c) s4 = fma(__ldg(D + (ai + y) * nao + ak + c), Vr(y, x, c, d), s4);
@@ -352,6 +390,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
       auto Vat = [&](auto x, auto b, auto c, auto d) -> double { return V[((x * NB + b) * NC + c) * ND + d]; };
       sfor<NA>([&](auto x) {
         sfor<NC>([&](auto c) {   // K_ik
+          if (((x * NC + c) & (S - 1)) != sub) return;
           double s1 = 0.0;
           sfor<NB>([&](auto b) {
             sfor<ND>([&](auto d) { s1 = fma(__ldg(D + (aj + b) * nao + al + d), Vat(x, b, c, d), s1); });
@@ -359,6 +398,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           atomicAdd(K + (ai + x) * nao + ak + c, w * s1);
         });
         sfor<ND>([&](auto d) {   // K_il
+          if (((x * ND + d) & (S - 1)) != sub) return;
           double s2 = 0.0;
           sfor<NB>([&](auto b) {
             sfor<NC>([&](auto c) { s2 = fma(__ldg(D + (aj + b) * nao + ak + c), Vat(x, b, c, d), s2); });
@@ -368,6 +408,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
       });
       sfor<NB>([&](auto x) {
         sfor<NC>([&](auto c) {   // K_jk
+          if (((x * NC + c) & (S - 1)) != sub) return;
           double s3 = 0.0;
           sfor<NA>([&](auto y) {
             sfor<ND>([&](auto d) { s3 = fma(__ldg(D + (ai + y) * nao + al + d), Vat(y, x, c, d), s3); });
@@ -375,6 +416,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           atomicAdd(K + (aj + x) * nao + ak + c, w * s3);
         });
         sfor<ND>([&](auto d) {   // K_jl
+          if (((x * ND + d) & (S - 1)) != sub) return;
           double s4 = 0.0;
           sfor<NA>([&](auto y) {
             sfor<NC>([&](auto c) { s4 = fma(__ldg(D + (ai + y) * nao + ak + c), Vat(y, x, c, d), s4); });
@@ -386,15 +428,42 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
   }
 }
 
+// How many lanes share a quartet (log2, over the bra and the ket primitive pairs). A launch of few quartets
+// of a contracted class is bound by the chain of primitive quartets that one thread runs (1.8 us each for
+// [ss|ss]), not by the FP64 pipe: its time is taken as the chain's work, times the number of times the
+// launch's lanes exceed kSatThreads, from where on the pipe is busy and lanes that idle in a partial round
+// of primitives cost as much as working ones. Measured: one-shot 4-center call on 2 atoms 77.1 -> 23.0 ms,
+// on 6 atoms 87.5 -> 26.0 ms, density fitting of 4 atoms 11.8 -> 6.1 ms, 8-molecule batched exchange
+// 163 -> 113 ms; launches of more than 24,000 quartets keep one lane each and their time. ck / cb: FP64 operations per primitive quartet and per bra
+// transform; cr: per step of the lanes' reduction.
+constexpr double kSatThreads = 152 * 160.0;
+inline void split_of(int64_t nq, int Kb, int Kk, double ck, double cb, double cr, int* lb, int* lk) {
+  double best = 1e300;
+  *lb = *lk = 0;
+  for (int ls = 0; ls <= 5; ++ls)
+    for (int b = 0; b <= ls; ++b) {
+      const int k = ls - b;
+      if ((b && (1 << b) >= 2 * Kb) || (k && (1 << k) >= 2 * Kk)) continue;
+      const double rounds = (Kb + (1 << b) - 1) >> b, per = (Kk + (1 << k) - 1) >> k;
+      const double chain = rounds * (per * ck + cb) + ls * cr;
+      const double t = chain * std::max(1.0, (double)nq * (1 << ls) / kSatThreads);
+      if (t < 0.97 * best) { best = t; *lb = b; *lk = k; }
+    }
+}
+
 template <int LA, int LB, int LC, int LD>
-cudaError_t launch_reg_class(const QuartetLaunch& a, cudaStream_t s) {
+cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
   constexpr bool XS = !reg_eligible(LA, LB, LC, LD);
   constexpr int bs = XS ? kXsBlock : 128;
   constexpr int Nk = ncart(LC) * ncart(LD);
   // shared memory per block: [p|cd] (and, with the digestion epilogue, the shellset) of every thread
   constexpr size_t shm_x = XS ? (size_t)nherm(LA + LB) * Nk * kXsBlock * sizeof(double) : 0;
   constexpr size_t shm_d = XS ? (size_t)ncart(LA) * ncart(LB) * Nk * kXsBlock * sizeof(double) + shm_x : 0;
-  const int64_t grid = (a.nq + bs - 1) / bs;
+  QuartetLaunch a = a0;
+  constexpr double ck = reg_body_size(LA, LB, LC, LD, false) + 8.0 * (LA + LB + LC + LD + 1) + 80.0;
+  constexpr double cb = reg_body_size(LA, LB, LC, LD) - reg_body_size(LA, LB, LC, LD, false);
+  split_of(a.nq, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
+  const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   if constexpr (shm_d > 48 * 1024) {
     // opt in to more than 48 KB of dynamic shared memory, once per instance and device
