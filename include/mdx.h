@@ -170,7 +170,10 @@ mdx_status mdx_eri3_sph(mdx_ctx* ctx, const mdx_basis* aux, const mdx_basis* orb
  * evaluated repeatedly and its launches enqueued without host
  * synchronisation or allocation (e.g. inside a captured CUDA graph).
  * The basis descriptors' device arrays must stay valid until the batch is
- * destroyed; the batch keeps its own copies of the index data. */
+ * destroyed; the batch keeps its own copies of the index data. The per-class
+ * launches of a run are spread over the caller's stream and the context's
+ * internal streams, ordered after the work already queued on the caller's
+ * stream, which waits for all of them. */
 typedef struct mdx_batch mdx_batch;
 
 /* Prepare the quartets of mdx_eri4 (same arguments, without screening
@@ -278,7 +281,7 @@ mdx_status mdx_schwarz(mdx_ctx* ctx, const mdx_basis* basis, const int32_t* pair
  *   E_x = alpha sum_ik D_ik K_ik = alpha sum_ijkl D_ik D_jl (ij|kl) of the
  *   screened K (alpha = -1 for a closed-shell D = C C^T), or NULL. Synchronises `stream` (screening counts) and on return K is
  *   complete. Pairs absent from the list contribute nothing. The per-class
- *   integral launches are spread over `stream` and three internal streams of
+ *   integral launches are spread over `stream` and the internal streams of
  *   the context, each ordered after the work already queued on `stream`, and
  *   `stream` waits for all of them before K <- K + K^T. */
 mdx_status mdx_exchange(mdx_ctx* ctx, const mdx_basis* basis, const int32_t* pairs, const double* Q, int64_t n_pairs,

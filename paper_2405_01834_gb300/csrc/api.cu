@@ -49,8 +49,12 @@ struct mdx_ctx {
   std::vector<std::unique_ptr<Plan>> retired;   // replaced plans, kept alive for batches that use them
   int64_t last_quartets = 0;
   cublasHandle_t cublas = nullptr;        // materialized-Hermite path only, created on first use
-  // auxiliary streams for independent per-class launches (created on first use)
-  static constexpr int kAux = 3;
+  // auxiliary streams for independent per-class launches. The classes of a molecule are chains of dependent
+  // FP64 operations on few SMs, so their times overlap almost fully: one-shot 4-center call on 6 atoms (81
+  // launches) 26.0 ms on one stream, 8.3 on eight; density fitting of 4 atoms (105 launches) 6.13 -> 2.54 ms;
+  // 8-molecule batched exchange 113 -> 73 ms; gradient of 3 atoms 199 ms on four streams, 162 on eight. The
+  // hardware runs 8 queues by default, hence 7 beside the caller's.
+  static constexpr int kAux = 7;
   cudaStream_t aux[kAux] = {};
   cudaEvent_t ev_fork = nullptr, ev_join[kAux] = {};
 };
@@ -235,6 +239,7 @@ struct mdx_batch {
   int64_t nxg = 0;                // doubles allocated at xg
   struct Range { Plan* plan; int64_t begin, count; ClassKey key; Plan* splan; int grid; };
   std::vector<Range> ranges;
+  std::vector<std::pair<double, int32_t>> order;   // (model FLOPs, range), heaviest first: launch order
   std::vector<int64_t> qorig;     // caller index of each class-sorted quartet
   double model_flops = 0.0;
   double exec_fma = 0.0;
@@ -264,7 +269,8 @@ struct mdx_xbatch {
   std::vector<QuartetLaunch> launches, plaunches;
   std::vector<ClassKey> lkey;          // class of each per-class launch
   std::vector<double> lflops;          // its Table-1 model FLOPs
-  std::vector<int32_t> reg_launches;   // per-class launches that run a register kernel
+  std::vector<char> is_reg;            // per-class launches that run a register kernel
+  std::vector<std::pair<double, int32_t>> order;   // (model FLOPs, launch), heaviest first: launch order
   QuartetLaunch* d_plaunches = nullptr;
   WorkItem* items = nullptr;
   WorkItem* items_team = nullptr;
@@ -307,41 +313,53 @@ mdx_status dev_upload(mdx_ctx* c, const std::vector<T>& v, T** out, cudaStream_t
   return MDX_OK;
 }
 
-// Independent launches (one per class, each summing into K or the gradient
-// with atomics) spread over the caller's stream and the context's auxiliary
-// streams, so that launches too small to fill the GPU overlap. fork() makes
-// every auxiliary stream wait for the work enqueued on the caller's stream so
-// far (plan uploads included); pick() takes the stream with the least work
-// assigned; join() makes the caller's stream wait for all of them.
+// Independent launches (one per class, each writing its own output or summing
+// into K or the gradient with atomics) spread over the caller's stream and the
+// context's auxiliary streams, so that launches too small to fill the GPU
+// overlap. fork(launches) makes the auxiliary streams that so many launches can
+// use wait for the work enqueued on the caller's stream so far (plan uploads
+// included); pick() takes the stream with the least work assigned; join()
+// makes the caller's stream wait for all of them. While a stream capture that
+// the caller's stream does not belong to holds an auxiliary stream (a caller
+// that captures on one stream and launches on another), everything stays on
+// the caller's stream.
 struct Fanout {
   mdx_ctx* c;
   cudaStream_t s;
+  int n = 0;   // auxiliary streams in use
   double load[mdx_ctx::kAux + 1] = {};
   cudaStream_t stream(int i) const { return i == 0 ? s : c->aux[i - 1]; }
-  cudaError_t fork() {
-    if (!c->ev_fork) {
-      for (int i = 0; i < mdx_ctx::kAux; ++i) {
-        cudaError_t e = c->aux[i] ? cudaSuccess : cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking);
-        if (e == cudaSuccess && !c->ev_join[i]) e = cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
-      }
-      const cudaError_t e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-      if (e != cudaSuccess) return e;
+  static cudaError_t capture_id(cudaStream_t st, unsigned long long* id) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    *id = 0;
+    const cudaError_t e = cudaStreamGetCaptureInfo(st, &status, id);
+    if (status == cudaStreamCaptureStatusNone) *id = 0;
+    return e;
+  }
+  cudaError_t fork(size_t launches) {
+    const int want = (int)std::min<size_t>(mdx_ctx::kAux, launches > 0 ? launches - 1 : 0);
+    if (want == 0) return cudaSuccess;
+    unsigned long long own = 0, other = 0;
+    cudaError_t e = capture_id(s, &own);
+    for (int i = 0; i < want && e == cudaSuccess; ++i) {
+      e = capture_id(c->aux[i], &other);
+      if (e == cudaSuccess && other != 0 && other != own) return cudaSuccess;
     }
-    cudaError_t e = cudaEventRecord(c->ev_fork, s);
-    for (int i = 0; i < mdx_ctx::kAux && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(c->aux[i], c->ev_fork, 0);
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev_fork, s);
+    for (int i = 0; i < want && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(c->aux[i], c->ev_fork, 0);
+    if (e == cudaSuccess) n = want;
     return e;
   }
   int pick(double work) {
     int best = 0;
-    for (int i = 1; i <= mdx_ctx::kAux; ++i)
+    for (int i = 1; i <= n; ++i)
       if (load[i] < load[best]) best = i;
     load[best] += work;
     return best;
   }
   cudaError_t join() {
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < mdx_ctx::kAux && e == cudaSuccess; ++i) {
+    for (int i = 0; i < n && e == cudaSuccess; ++i) {
       e = cudaEventRecord(c->ev_join[i], c->aux[i]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join[i], 0);
     }
@@ -456,9 +474,13 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
       }
     }
     B->ranges.push_back({plan, b, cnt, kv.first, splan, grid});
-    B->model_flops += model_flops_class(kv.first, sph) * (double)cnt;
+    const double model = model_flops_class(kv.first, sph) * (double)cnt;
+    B->order.emplace_back(model, (int32_t)B->ranges.size() - 1);
+    B->model_flops += model;
     B->exec_fma += fma * (double)cnt;
   }
+  std::stable_sort(B->order.begin(), B->order.end(),
+                   [](const std::pair<double, int32_t>& x, const std::pair<double, int32_t>& y) { return x.first > y.first; });
   B->njobs = (int64_t)jobs.size();
   if (call_ws) {
     if ((st = upload(c, "call_jobs", jobs, &B->jobs, s)) != MDX_OK) return st;
@@ -499,7 +521,10 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
 }
 
 // Enqueue the whole hot path of a batch: pair records, then one quartet
-// kernel per class. No host synchronisation, no allocation.
+// kernel per class, heaviest first, spread over `s` and the context's
+// auxiliary streams (the classes of a molecule are small launches that leave
+// most SMs idle one by one). Classes of the solid-harmonic team kernel share
+// one staging area and stay on `s`. No host synchronisation, no allocation.
 mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cudaStream_t s) {
   int32_t nl = 0;
   cudaError_t e = launch_pair_records(B->b0, B->b1, B->jobs, B->njobs, B->recs, B->recs_s, c->d_err, s);
@@ -510,7 +535,11 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
     if (e != cudaSuccess) return cuda_fail(c, e, "screened-out shellsets");
     ++nl;
   }
-  for (auto& r : B->ranges) {
+  Fanout fan{c, s};
+  e = fan.fork(B->ranges.size());
+  for (size_t i = 0; i < B->order.size() && e == cudaSuccess; ++i) {
+    auto& r = B->ranges[B->order[i].second];
+    if (r.count == 0) continue;
     QuartetLaunch a{};
     a.plan = r.plan->d;
     a.nq = r.count;
@@ -527,26 +556,28 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
     if (B->sph && r.splan) {   // solid harmonics folded into the transforms
       a.plan = r.splan->d;
       a.sph_scratch = B->xg;
+      fan.load[0] += B->order[i].first;
       e = launch_quartets_sph(a, r.grid, s);
-      if (e != cudaSuccess) return cuda_fail(c, e, "solid-harmonic quartet kernel launch");
-      if (r.count > 0) ++nl;
+      ++nl;
       continue;
     }
+    const cudaStream_t rs = fan.stream(fan.pick(B->order[i].first));
     if (B->sph) {              // Cartesian shellsets, then the index-by-index transform
       a.qout = B->cqoff + r.begin;
       a.out = B->cart;
     }
-    e = launch_quartets(a, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "quartet kernel launch");
-    if (r.count > 0) ++nl;
-    if (B->sph) {
+    e = launch_quartets(a, rs);
+    ++nl;
+    if (B->sph && e == cudaSuccess) {
       SphLaunch t{r.key.la, r.key.lb, r.key.lc, r.key.ld, r.count, B->cart, B->cqoff + r.begin, out,
                   B->qoff + r.begin};
-      e = launch_cart2sph(t, s);
-      if (e != cudaSuccess) return cuda_fail(c, e, "solid-harmonic transform");
-      if (r.count > 0) ++nl;
+      e = launch_cart2sph(t, rs);
+      ++nl;
     }
   }
+  const cudaError_t ej = fan.join();   // also after a failed launch: the streams must not stay forked
+  if (e == cudaSuccess) e = ej;
+  if (e != cudaSuccess) return cuda_fail(c, e, "quartet kernel launch");
   if (nlaunch) *nlaunch = nl;
   return MDX_OK;
 }
@@ -705,6 +736,15 @@ mdx_status mdx_create(mdx_ctx** ctx, int device) {
     return MDX_ECUDA;
   if (cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess) return MDX_ENOMEM;
   if (cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess) return MDX_ECUDA;
+  bool streams = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < mdx_ctx::kAux && streams; ++i)
+    streams = cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&c->ev_join[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!streams) {
+    cudaGetLastError();
+    mdx_destroy(c.release());
+    return MDX_ECUDA;
+  }
   *ctx = c.release();
   return MDX_OK;
 }
@@ -1527,7 +1567,7 @@ mdx_status mdx_exchange(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs
                        return x.first > y.first;
                      });
     Fanout fan{c, s};
-    e = fan.fork();
+    e = fan.fork(jobs_k.size());
     for (size_t i = 0; i < jobs_k.size() && e == cudaSuccess; ++i)
       e = launch_quartets(jobs_k[i].second, fan.stream(fan.pick(jobs_k[i].first)));
     const cudaError_t ej = fan.join();
@@ -1733,24 +1773,22 @@ mdx_status mdx_exchange_grad(mdx_ctx* c, const mdx_basis* basis, const int32_t* 
         GradJob g{a, model_flops_class(key) * (double)a.nq, 0, 0};
         if (plan->d.reg) {
           // register kernel: shifted shellsets to workspace (back to back), then the
-          // gradient contraction, in chunks of at most 1 GiB of shellsets
+          // gradient contraction, in chunks of at most 512 MiB of shellsets per stream
           g.per = (int64_t)plan->d.Nb * plan->d.Nk;
-          g.chunk = std::max<int64_t>(1, std::min<int64_t>(a.nq, (int64_t(1) << 27) / g.per));
+          g.chunk = std::max<int64_t>(1, std::min<int64_t>(a.nq, (int64_t(1) << 26) / g.per));
           ws_doubles = std::max(ws_doubles, g.chunk * g.per);
         }
         gjobs.push_back(g);
       }
     }
   // one shellset workspace per stream
-  static const char* const kWsName[mdx_ctx::kAux + 1] = {"g_shellsets0", "g_shellsets1", "g_shellsets2",
-                                                          "g_shellsets3"};
   double* ws[mdx_ctx::kAux + 1] = {};
   if (ws_doubles > 0)
     for (int i = 0; i <= mdx_ctx::kAux; ++i)
-      if ((st = ensure(c, kWsName[i], (size_t)ws_doubles, &ws[i], s)) != MDX_OK) return st;
+      if ((st = ensure(c, ("g_shellsets" + std::to_string(i)).c_str(), (size_t)ws_doubles, &ws[i], s)) != MDX_OK) return st;
   std::stable_sort(gjobs.begin(), gjobs.end(), [](const GradJob& x, const GradJob& y) { return x.work > y.work; });
   Fanout fan{c, s};
-  e = fan.fork();
+  e = fan.fork(gjobs.size());
   for (size_t j = 0; j < gjobs.size() && e == cudaSuccess; ++j) {
     const GradJob& g = gjobs[j];
     const int si = fan.pick(g.work);
@@ -2154,8 +2192,11 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
           cost.push_back(pp->exec_fma * cnt);
           item_reg.push_back(reg_class);
         }
-        if (reg_class) X->reg_launches.push_back((int32_t)(X->launches.size() - 1));
+        X->is_reg.push_back(reg_class);
+        X->order.emplace_back(X->lflops.back(), (int32_t)(X->launches.size() - 1));
       }
+    std::stable_sort(X->order.begin(), X->order.end(),
+                     [](const std::pair<double, int32_t>& x, const std::pair<double, int32_t>& y) { return x.first > y.first; });
     // heaviest items first (the queue hands them out in order)
     std::vector<size_t> iorder(items.size());
     for (size_t i = 0; i < iorder.size(); ++i) iorder[i] = i;
@@ -2216,25 +2257,26 @@ mdx_status mdx_xbatch_run(mdx_ctx* c, mdx_xbatch* xb, int32_t persistent, int32_
       PersistLaunch pl{xb->d_plaunches, xb->items, xb->nitems, xb->counter};
       if (e == cudaSuccess) e = launch_persistent(pl, xb->smem, xb->grid, s);
       ++nl;
-    } else if (persistent == 2) {
-      // register-kernel classes one launch each, then one persistent launch for the rest
-      for (int32_t i : xb->reg_launches) {
-        e = launch_quartets(xb->launches[i], s);
-        if (e != cudaSuccess) break;
-        ++nl;
-      }
-      if (e == cudaSuccess && xb->nitems_team > 0) {
+    } else {
+      // one launch per class (mode 2: per register-kernel class, the rest in one persistent launch first),
+      // heaviest first, spread over the streams
+      Fanout fan{c, s};
+      e = fan.fork(xb->order.size() + (persistent == 2 ? 1 : 0));
+      if (e == cudaSuccess && persistent == 2 && xb->nitems_team > 0) {
         e = cudaMemsetAsync(xb->counter, 0, sizeof(unsigned long long), s);
         PersistLaunch pl{xb->d_plaunches, xb->items_team, xb->nitems_team, xb->counter};
         if (e == cudaSuccess) e = launch_persistent(pl, xb->smem_team, xb->grid_team, s);
+        fan.load[0] = 1e300;   // nothing queues behind it
         ++nl;
       }
-    } else {
-      for (const QuartetLaunch& a : xb->launches) {
-        e = launch_quartets(a, s);
-        if (e != cudaSuccess) break;
+      for (size_t i = 0; i < xb->order.size() && e == cudaSuccess; ++i) {
+        const QuartetLaunch& a = xb->launches[xb->order[i].second];
+        if (persistent == 2 && !xb->is_reg[xb->order[i].second]) continue;
+        e = launch_quartets(a, fan.stream(fan.pick(xb->order[i].first)));
         ++nl;
       }
+      const cudaError_t ej = fan.join();   // also after a failed launch: the streams must not stay forked
+      if (e == cudaSuccess) e = ej;
     }
   }
   if (e == cudaSuccess) e = launch_multi_k(xb->molK, xb->molnao, xb->nmol, xb->max_nao, false, s);

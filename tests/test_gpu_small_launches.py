@@ -1,5 +1,8 @@
-"""Launches too small to fill the GPU: lanes that share a quartet's primitive pairs in the register kernel."""
+"""Launches too small to fill the GPU: lanes that share a quartet's primitive pairs in the register kernel, and
+per-class launches spread over several streams (also inside a stream capture)."""
+import numpy as np
 import pytest
+import torch
 
 import oracle
 from oracle import parity
@@ -24,4 +27,38 @@ def test_lanes_sharing_a_quartet(lq, K):
         parity.check(part.cpu().numpy(), ref[: roff[n]], roff[: n + 1], "%s K=%s n=%d" % (lq, K, n),
                      parity.Eri4Evaluator(b, q[:n]))
     eng.sync()
+    eng.close()
+
+
+def test_multi_class_batch_in_a_capture():
+    """A captured multi-class run replays to the same bits; a run of another batch on another stream while the
+    capture holds the context's streams keeps its own results."""
+    b = inputs.small_molecule(n_atoms=3)
+    q = inputs.unique_quartets(b.n_shells)
+    eng, db = mdx.Engine(0), mdx.DeviceBasis(b)
+    b1, b2 = eng.batch_eri4(db, q), eng.batch_eri4(db, q[::3])
+    o1, o2 = (torch.zeros(x.total, dtype=torch.float64, device="cuda") for x in (b1, b2))
+    b1.run(o1)
+    b2.run(o2)
+    torch.cuda.synchronize()
+    want1, want2 = o1.clone(), o2.clone()
+    o1.zero_()
+    o2.zero_()
+    torch.cuda.synchronize()
+    side, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        b1.run(o1)
+        with torch.cuda.stream(side):
+            b2.run(o2)
+        b1.run(o1)
+    torch.cuda.synchronize()
+    assert torch.equal(o2, want2) and not o1.any()
+    for _ in range(2):
+        o1.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(o1, want1)
+    eng.sync()
+    b1.close()
+    b2.close()
     eng.close()
