@@ -553,6 +553,7 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
     a.rprog_off = c->d_rprog_off;
     a.out = out;
     a.err = c->d_err;
+    a.concurrent = fan.n + 1;
     if (B->sph && r.splan) {   // solid harmonics folded into the transforms
       a.plan = r.splan->d;
       a.sph_scratch = B->xg;
@@ -1568,6 +1569,7 @@ mdx_status mdx_exchange(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs
                      });
     Fanout fan{c, s};
     e = fan.fork(jobs_k.size());
+    for (size_t i = 0; i < jobs_k.size(); ++i) jobs_k[i].second.concurrent = fan.n + 1;
     for (size_t i = 0; i < jobs_k.size() && e == cudaSuccess; ++i)
       e = launch_quartets(jobs_k[i].second, fan.stream(fan.pick(jobs_k[i].first)));
     const cudaError_t ej = fan.join();
@@ -1790,7 +1792,8 @@ mdx_status mdx_exchange_grad(mdx_ctx* c, const mdx_basis* basis, const int32_t* 
   Fanout fan{c, s};
   e = fan.fork(gjobs.size());
   for (size_t j = 0; j < gjobs.size() && e == cudaSuccess; ++j) {
-    const GradJob& g = gjobs[j];
+    GradJob& g = gjobs[j];
+    g.a.concurrent = fan.n + 1;
     const int si = fan.pick(g.work);
     const cudaStream_t gs = fan.stream(si);
     if (g.chunk == 0) {
@@ -2270,7 +2273,8 @@ mdx_status mdx_xbatch_run(mdx_ctx* c, mdx_xbatch* xb, int32_t persistent, int32_
         ++nl;
       }
       for (size_t i = 0; i < xb->order.size() && e == cudaSuccess; ++i) {
-        const QuartetLaunch& a = xb->launches[xb->order[i].second];
+        QuartetLaunch a = xb->launches[xb->order[i].second];
+        a.concurrent = fan.n + 1;
         if (persistent == 2 && !xb->is_reg[xb->order[i].second]) continue;
         e = launch_quartets(a, fan.stream(fan.pick(xb->order[i].first)));
         ++nl;

@@ -161,6 +161,29 @@ __device__ __forceinline__ void team_sync(unsigned mask) {
   }
 }
 
+// Thread-block cluster: barrier over all its threads, its size, this block's rank, and a double at the same
+// shared-memory offset of block `rank`.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ int cluster_size() {
+  int n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return n;
+}
+__device__ __forceinline__ int cluster_rank() {
+  int r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ double cluster_read(const double* p, int rank) {
+  uint32_t addr;
+  double v;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ int d_tet(int n) { return n < 0 ? 0 : n * (n + 1) * (n + 2) / 6; }
 __device__ __forceinline__ int d_tri(int n) { return n < 0 ? 0 : n * (n + 1) / 2; }
 
@@ -625,6 +648,12 @@ __device__ __forceinline__ void bra_b23(const PlanDev& P, double* ws, int o_C1, 
   }
 }
 
+// The share of a quartet's primitive pairs that one team works on: bra pairs b, b + nb, ... and of each the
+// ket pairs k, k + nk, ...
+struct PrimPart {
+  int b, nb, k, nk;
+};
+
 // R of primitive quartet i from the cache into R0, where the k1 programs read it.
 __device__ __forceinline__ void load_cached_R(const PlanDev& P, double* ws, int i, int tl) {
   const int nR = d_tet(P.L + 1);
@@ -640,11 +669,11 @@ __device__ __forceinline__ void load_cached_R(const PlanDev& P, double* ws, int 
 // groups would otherwise compute each R once per group.
 template <bool CTA>
 __device__ __forceinline__ void fill_R_cache(const QuartetLaunch& a, double* ws, int64_t bra0, int64_t ket0, int pb0,
-                                             int pb1, int tl, unsigned mask) {
+                                             int pb1, int tl, unsigned mask, PrimPart part = PrimPart{0, 1, 0, 1}) {
   const PlanDev& P = a.plan;
   const int nR = d_tet(P.L + 1);
-  for (int pb = pb0; pb < pb1; ++pb)
-    for (int pk = 0; pk < P.Kk; ++pk) {
+  for (int pb = pb0 + part.b; pb < pb1; pb += part.nb)
+    for (int pk = part.k; pk < P.Kk; pk += part.nk) {
       load_record(ws + P.o_recb, a.recs + bra0 + (int64_t)pb * P.recb, P.recb, tl, P.T);
       load_record(ws + P.o_reck, a.recs_signed + ket0 + (int64_t)pk * P.reck, P.reck, tl, P.T);
       team_sync<CTA>(mask);   // also orders the previous table's copy before compute_R rewrites R0
@@ -658,9 +687,13 @@ __device__ __forceinline__ void fill_R_cache(const QuartetLaunch& a, double* ws,
 // The work of one team on one shell quartet q (all groups, all primitives,
 // store / digestion / gradient epilogue). Inactive teams run the same control
 // flow on a shadow quartet (so that barriers match) and write nothing global.
-template <bool CTA>
+//
+// part: the team's share of the primitive pairs. Every epilogue is linear in the shellset, so the teams that
+// share a quartet digest or contract their own partial shellsets; with the store epilogue they are the blocks
+// of a cluster (CL), which add up their OUT regions through distributed shared memory, group by group.
+template <bool CTA, bool CL = false>
 __device__ __forceinline__ void quartet_body(const QuartetLaunch& a, double* ws, int64_t q, bool active, int tl,
-                                             unsigned mask) {
+                                             unsigned mask, const PrimPart part = PrimPart{0, 1, 0, 1}) {
   const PlanDev& P = a.plan;
   const int T = P.T;
   const int2 qp = a.qpairs[q];
@@ -673,19 +706,20 @@ __device__ __forceinline__ void quartet_body(const QuartetLaunch& a, double* ws,
     team_sync<CTA>(mask);
     compute_R<CTA>(a, ws, tl, mask);
   } else if (P.cache_R == 2) {
-    fill_R_cache<CTA>(a, ws, bra0, ket0, 0, Kb, tl, mask);
+    fill_R_cache<CTA>(a, ws, bra0, ket0, 0, Kb, tl, mask, part);
   }
   // qout == nullptr: shellsets back to back, N_b N_k doubles each
   double* outq = a.D ? nullptr : a.out + (a.qout ? a.qout[q] : q * (int64_t)P.Nb * P.Nk);
   // store epilogue: b23 of the last bra primitive writes the shellset to global
   // memory itself (no OUT pass, no barrier after it)
-  const bool direct = !a.D && !a.grad;
+  const bool direct = !CL && !a.D && !a.grad;
   for (int g = 0; g < P.ngroups; ++g) {
     const Group grp = P.groups[g];
     const int ncols = grp.ncols;
-    for (int pb = 0; pb < Kb; ++pb) {
+    for (int pb = part.b; pb < Kb; pb += part.nb) {
+      const bool last_b = pb + part.nb >= Kb;
       if (P.cache_R != 1) load_record(ws + P.o_recb, a.recs + bra0 + (int64_t)pb * P.recb, P.recb, tl, T);
-      for (int pk = 0; pk < Kk; ++pk) {
+      for (int pk = part.k; pk < Kk; pk += part.nk) {
         if (P.cache_R != 1) {
           load_record(ws + P.o_reck, a.recs_signed + ket0 + (int64_t)pk * P.reck, P.reck, tl, T);
           if (P.cache_R == 2) load_cached_R(P, ws, pb * Kk + pk, tl);
@@ -698,19 +732,32 @@ __device__ __forceinline__ void quartet_body(const QuartetLaunch& a, double* ws,
         }
         run_step(P.kprog + grp.k2_off, grp.k2_n, ws, tl, T, false);
         team_sync<CTA>(mask);
-        run_step(P.kprog + grp.k3_off, grp.k3_n, ws, tl, T, pk > 0);
+        run_step(P.kprog + grp.k3_off, grp.k3_n, ws, tl, T, pk > part.k);
         team_sync<CTA>(mask);
       }
       bra_b1(P, ws, P.o_X, P.o_C1, P.c1size, ncols, tl, T);
       team_sync<CTA>(mask);
-      bra_b23(P, ws, P.o_C1, P.c1size, P.o_OUT, ncols, pb > 0, direct && pb == Kb - 1, outq,
+      bra_b23(P, ws, P.o_C1, P.c1size, P.o_OUT, ncols, pb > part.b, direct && last_b, outq,
               P.colmap + grp.col_off, P.Nk, active, tl, T);
       // Barrier before the next writer of what b23 reads: the bra record (reloaded
       // per bra primitive unless the class has one primitive quartet) or OUT (read
       // by other lanes in the digestion / gradient epilogue). C1 is overwritten by
       // the next b1 only after the k-step barriers.
-      if (P.cache_R != 1 || (!direct && pb == Kb - 1)) team_sync<CTA>(mask);
+      if (P.cache_R != 1 || (!direct && last_b)) team_sync<CTA>(mask);
     }
+    if constexpr (CL) {
+      // every block of the cluster adds up its share of the group's columns over all blocks and stores it
+      cluster_sync();
+      const int n = cluster_size(), tot = P.Nb * ncols;
+      const uint16_t* cm = P.colmap + grp.col_off;
+      for (int e = cluster_rank() * T + tl; e < tot; e += n * T) {
+        double v = 0.0;
+        for (int r = 0; r < n; ++r) v += cluster_read(ws + P.o_OUT + e, r);
+        const int ab = e / ncols, col = e - ab * ncols;
+        if (active) outq[(int64_t)ab * P.Nk + cm[col]] = v;
+      }
+      cluster_sync();   // the next group rewrites OUT
+    } else
     if (a.grad) {
       grad_group<CTA>(a, ws, grp, qp, tl, T, active, mask);
       team_sync<CTA>(mask);
@@ -725,7 +772,7 @@ __device__ __forceinline__ void quartet_body(const QuartetLaunch& a, double* ws,
   if (direct) team_sync<CTA>(mask);
 }
 
-template <bool CTA>
+template <bool CTA, bool CL>
 __global__ void __launch_bounds__(CTA ? 1024 : 128) k_quartets(const QuartetLaunch a) {
   extern __shared__ __align__(16) double smem[];
   const PlanDev& P = a.plan;
@@ -741,10 +788,12 @@ __global__ void __launch_bounds__(CTA ? 1024 : 128) k_quartets(const QuartetLaun
     const int live = blockDim.x - wbase;
     if (live < 32) mask = (1u << live) - 1u;
   }
-  int64_t q = (int64_t)blockIdx.x * P.teams_per_cta + team;
+  // parts consecutive blocks (with CL: the blocks of one cluster) share the same quartets' primitive pairs
+  const int parts = a.part_b * a.part_k, pi = (int)(blockIdx.x % (unsigned)parts);
+  int64_t q = (int64_t)(blockIdx.x / (unsigned)parts) * P.teams_per_cta + team;
   const bool active = q < a.nq;
   if (!active) q = a.nq - 1;   // idle teams shadow the last quartet and store nothing
-  quartet_body<CTA>(a, ws, q, active, tl, mask);
+  quartet_body<CTA, CL>(a, ws, q, active, tl, mask, PrimPart{pi / a.part_k, a.part_b, pi % a.part_k, a.part_k});
 }
 
 // One quartet over real solid harmonics (Eqs. solid2herm-1/2: the
@@ -1022,6 +1071,33 @@ static const RegPart kRegParts[] = {launch_reg_part00, launch_reg_part01, launch
                                     launch_reg_part08, launch_reg_part09, launch_reg_part10, launch_reg_part11,
                                     launch_reg_part12, launch_reg_part13, launch_reg_part14};
 
+// How many teams share a quartet's bra and ket primitive pairs. A launch of few quartets of a contracted
+// class is bound by one team's chain of barrier-separated steps over its primitive quartets (about 10 us each
+// at L = 7), so its time is taken as the chain's, times the number of rounds in which the launch's teams
+// exceed those that the SMs hold with the FP64 pipe kept busy (its share of them where several launches run
+// side by side). A split over the ket pairs repeats the bra steps, and every split the epilogue. Teams that
+// store their shellset add it up inside a cluster (portable size: 8 blocks) and need the OUT region.
+// Measured: one-shot 4-center call on 2 atoms 5.17 -> 2.04 ms ([dd|dd] K = 81: one team's 0.85 ms chain in
+// 8 parts); exchange of 5 atoms 90 -> 77 ms and 8-molecule batched exchange 73 -> 63 ms, where without the
+// share of the SMs the repeated work made the gradient of 3 atoms slower (162 -> 173 ms; with it 149).
+static void team_parts(const QuartetLaunch& a, int* nb, int* nk) {
+  const PlanDev& P = a.plan;
+  *nb = *nk = 1;
+  if (P.Kb * P.Kk == 1 || !P.has_out) return;
+  const bool store = !a.D && !a.grad;
+  const int64_t cta = (int64_t)P.teams_per_cta * P.team_doubles * 8 + 1024, block = P.teams_per_cta * P.T;
+  const int64_t fit = std::min<int64_t>(228 * 1024 / cta, std::max<int64_t>(1, 512 / block));
+  const double sat = 152.0 * (double)std::max<int64_t>(1, fit) * P.teams_per_cta / std::max(1, a.concurrent);
+  const double ck = P.cost_k, cb = P.cost_b, ce = store ? 0.2 * P.cost_b : P.cost_b;
+  double best = 1e300;
+  for (int b = 1; b <= std::min(P.Kb, store ? 8 : 64); ++b)
+    for (int k = 1; k <= std::min(P.Kk, (store ? 8 : 64) / b); ++k) {
+      const double chain = (double)((P.Kb + b - 1) / b) * ((double)((P.Kk + k - 1) / k) * ck + cb) + ce;
+      const double t = chain * std::max(1.0, (double)a.nq * b * k / sat);
+      if (t < 0.95 * best) { best = t; *nb = b; *nk = k; }
+    }
+}
+
 cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s) {
   if (a.nq <= 0) return cudaSuccess;
   const PlanDev& P = a.plan;
@@ -1035,12 +1111,30 @@ cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s) {
       if (handled || e != cudaSuccess) return e;
     }
   }
-  const int64_t grid = (a.nq + P.teams_per_cta - 1) / P.teams_per_cta;
+  QuartetLaunch b = a;
+  team_parts(a, &b.part_b, &b.part_k);
+  const int parts = b.part_b * b.part_k;
+  const int64_t grid = (a.nq + P.teams_per_cta - 1) / P.teams_per_cta * parts;
   const int block = P.teams_per_cta * P.T;
   const size_t shm = (size_t)P.teams_per_cta * P.team_doubles * sizeof(double);
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
-  if (P.T > 32) k_quartets<true><<<(unsigned)grid, block, shm, s>>>(a);
-  else k_quartets<false><<<(unsigned)grid, block, shm, s>>>(a);
+  if (parts > 1 && !a.D && !a.grad) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)parts;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return P.T > 32 ? cudaLaunchKernelEx(&cfg, k_quartets<true, true>, b)
+                    : cudaLaunchKernelEx(&cfg, k_quartets<false, true>, b);
+  }
+  if (P.T > 32) k_quartets<true, false><<<(unsigned)grid, block, shm, s>>>(b);
+  else k_quartets<false, false><<<(unsigned)grid, block, shm, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -1383,9 +1477,13 @@ cudaError_t kernel_attributes_init() {
     if (e != cudaSuccess) return e;
   }
   const int maxshm = 227 * 1024;
-  e = cudaFuncSetAttribute(k_quartets<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
+  e = cudaFuncSetAttribute(k_quartets<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_quartets<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
+  e = cudaFuncSetAttribute(k_quartets<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_quartets<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_quartets<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_quartets_sph<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
   if (e != cudaSuccess) return e;

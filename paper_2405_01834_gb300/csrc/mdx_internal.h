@@ -170,6 +170,7 @@ struct PlanDev {
   // lower Hermite term of its Cartesian expansion cancels), so the ket steps form only the rows |p| = l_a
   // and the bra step is OUT[m] = (2 zeta)^-l_a sum_a C_ma [a|cd] over those rows
   int32_t top_only;
+  float cost_k, cost_b;                  // a team's chain (clocks, roughly) per primitive quartet and per bra transform
   int64_t xg_doubles;                    // staging per team: Xg [Nk][hbp] then Yg [nc_c * nsd][hbp]
   const Group* groups;
   const StepEntry* kprog;

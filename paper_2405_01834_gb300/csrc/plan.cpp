@@ -655,6 +655,11 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
     }
     P.teams_per_cta = best;
   }
+  // a team's chain: a barrier-separated step costs some 500 clocks of load and barrier latency, and each of
+  // its lanes' multiply-adds about 24
+  const double nrec_k = P.cache_R == 2 ? 0.0 : P.ngroups;   // R levels inside the group loop
+  P.cost_k = (float)(500.0 * (nrec_k * (P.L + 2) + 4.0 * P.ngroups) + 24.0 * (fma_k + nrec_k * fma_r) / P.T);
+  P.cost_b = (float)(500.0 * 2.0 * P.ngroups + 24.0 * fma_b * P.Nk / P.T);
   if (P.T * P.teams_per_cta > 1024 || (long)P.teams_per_cta * P.team_doubles * 8 > 227 * 1024) {
     err = "team shape exceeds the CTA limits";
     return false;

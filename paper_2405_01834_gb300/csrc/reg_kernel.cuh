@@ -437,7 +437,8 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
 // 163 -> 113 ms; launches of more than 24,000 quartets keep one lane each and their time. ck / cb: FP64 operations per primitive quartet and per bra
 // transform; cr: per step of the lanes' reduction.
 constexpr double kSatThreads = 152 * 160.0;
-inline void split_of(int64_t nq, int Kb, int Kk, double ck, double cb, double cr, int* lb, int* lk) {
+inline void split_of(int64_t nq, int concurrent, int Kb, int Kk, double ck, double cb, double cr, int* lb, int* lk) {
+  const double sat = kSatThreads / std::max(1, concurrent);   // this launch's share of the SMs
   double best = 1e300;
   *lb = *lk = 0;
   for (int ls = 0; ls <= 5; ++ls)
@@ -446,7 +447,7 @@ inline void split_of(int64_t nq, int Kb, int Kk, double ck, double cb, double cr
       if ((b && (1 << b) >= 2 * Kb) || (k && (1 << k) >= 2 * Kk)) continue;
       const double rounds = (Kb + (1 << b) - 1) >> b, per = (Kk + (1 << k) - 1) >> k;
       const double chain = rounds * (per * ck + cb) + ls * cr;
-      const double t = chain * std::max(1.0, (double)nq * (1 << ls) / kSatThreads);
+      const double t = chain * std::max(1.0, (double)nq * (1 << ls) / sat);
       if (t < 0.97 * best) { best = t; *lb = b; *lk = k; }
     }
 }
@@ -462,7 +463,7 @@ cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
   QuartetLaunch a = a0;
   constexpr double ck = reg_body_size(LA, LB, LC, LD, false) + 8.0 * (LA + LB + LC + LD + 1) + 80.0;
   constexpr double cb = reg_body_size(LA, LB, LC, LD) - reg_body_size(LA, LB, LC, LD, false);
-  split_of(a.nq, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
+  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
   const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   if constexpr (shm_d > 48 * 1024) {

@@ -30,6 +30,23 @@ def test_lanes_sharing_a_quartet(lq, K):
     eng.close()
 
 
+# team-kernel classes (total angular momentum 7 and more, several column groups in the last): teams that share a
+# quartet's primitive pairs, summed inside a cluster (store) or digested one by one (exchange)
+@pytest.mark.parametrize("lq,K", [((2, 2, 2, 1), (3, 3, 3, 3)), ((3, 2, 2, 0), (1, 2, 1, 5)), ((2, 2, 2, 2), (2, 1, 2, 3)),
+                                  ((3, 3, 3, 3), (1, 2, 2, 1)), ((4, 1, 1, 1), (1, 7, 3, 1))])
+def test_teams_sharing_a_quartet(lq, K):
+    b, q = inputs.class_sweep(lq, n_bra=5, n_ket=7, seed=78, K=K)
+    eng, db = mdx.Engine(0), mdx.DeviceBasis(b)
+    assert eng.plan_info(*lq, K[0] * K[1], K[2] * K[3]).register_kernel == 0
+    ref, roff = oracle.eri4(b, q)
+    for n in (1, 3, len(q)):
+        v, off = eng.eri4(db, q[:n])
+        parity.check(v.cpu().numpy(), ref[: roff[n]], roff[: n + 1], "%s K=%s n=%d" % (lq, K, n),
+                     parity.Eri4Evaluator(b, q[:n]))
+    eng.sync()
+    eng.close()
+
+
 def test_multi_class_batch_in_a_capture():
     """A captured multi-class run replays to the same bits; a run of another batch on another stream while the
     capture holds the context's streams keeps its own results."""
