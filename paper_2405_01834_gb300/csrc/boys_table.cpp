@@ -44,6 +44,14 @@ std::vector<double> build_boys_table() {
       }
     }
   }
+  // last row: F_m(T) T^(m+1/2) for large T (the register kernel reads it instead of branching)
+  long double c = 0.886226925452758013649083741670572591L;   // sqrt(pi) / 2
+  for (int m = 0; m < kBoysOrders; ++m) {
+    double* row = tab.data() + (size_t)(kBoysNgrid - 1) * kBoysRow + (size_t)m * kBoysTerms;
+    row[0] = (double)c;
+    for (int k = 1; k < kBoysTerms; ++k) row[k] = 0.0;
+    c *= (long double)m + 0.5L;
+  }
   return tab;
 }
 

@@ -20,7 +20,8 @@ constexpr int kBoysOrders = kBoysMmax + 1;          // m = 0 .. kBoysMmax
 constexpr int kBoysRow = kBoysOrders * kBoysTerms;  // one grid point: [m][k]
 constexpr double kBoysInvH = 16.0;                  // grid spacing h = 1/16
 constexpr double kBoysTmax = 100.0;                 // asymptotic form above
-constexpr int kBoysNgrid = 1601 + 1;                // T0 = 0 .. 100 (+1 guard row)
+constexpr int kBoysNgrid = 1601 + 1;                // T0 = 0 .. 100, and a last row of the asymptotic constants:
+                                                    // coefficient 0 is Gamma(m+1/2)/2, the others 0
 
 // Builds the interpolation table [kBoysNgrid][kBoysOrders][kBoysTerms]
 // (row-major) in long double by downward recursion (see boys_table.cpp).
@@ -29,7 +30,7 @@ std::vector<double> build_boys_table();
 // ----------------------------------------------------------------- records
 // Primitive-pair record: header of kRecHeader doubles, then the three per-axis
 // E tables (x, y, z). Header: [0] zeta_p, [1] 1/zeta_p, [2..4] P, [5] prefactor
-// c_a c_b exp(-zeta_a zeta_b |A-B|^2 / zeta_p), [6], [7] unused.
+// c_a c_b exp(-zeta_a zeta_b |A-B|^2 / zeta_p), [6] the prefactor over zeta_p, [7] unused.
 constexpr int kRecHeader = 8;
 
 inline int etab_size(int la, int lb) {      // sum over a<=la, b<=lb of (a+b+1)

@@ -587,16 +587,21 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
         for (int ay = l - ax; ay >= 0; --ay) v.push_back({ax, ay, l - ax - ay});
       return v;
     };
+    // products Ex Ey Ez (a one-term table is the number 1)
+    auto eprod = [](int nx, int ny, int nz) {
+      const int axes = (nx > 1) + (ny > 1) + (nz > 1);
+      return axes < 2 ? 0 : nx * ny * nz + (axes == 3 ? nx * ny : 0);
+    };
     double ket = 0, bra = 0;
     for (auto& c : comps(key.lc))
       for (auto& d : comps(key.ld)) {
         const int nx = c[0] + d[0] + 1, ny = c[1] + d[1] + 1, nz = c[2] + d[2] + 1;
-        ket += nx * ny * nz + nx * ny + (double)nherm(P.Lb) * nx * ny * nz;
+        ket += eprod(nx, ny, nz) + (double)nherm(P.Lb) * nx * ny * nz;
       }
     for (auto& a : comps(key.la))
       for (auto& b : comps(key.lb)) {
         const int nx = a[0] + b[0] + 1, ny = a[1] + b[1] + 1, nz = a[2] + b[2] + 1;
-        bra += nx * ny * nz + nx * ny + (double)P.Nk * nx * ny * nz;
+        bra += eprod(nx, ny, nz) + (double)P.Nk * nx * ny * nz;
       }
     plan.exec_fma = key.Kb * key.Kk * (fma_r + 8.0 * (P.L + 1) + ket) + key.Kb * bra;
   }

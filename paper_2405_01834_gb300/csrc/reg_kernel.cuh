@@ -89,6 +89,29 @@ struct TArr<true, N> {
   __device__ __forceinline__ double& operator[](int i) { return p[i * kXsBlock]; }
 };
 
+// One step of Eq. r along an axis: X r1 + (i - 1) r2 for an entry of index i (no second term for i = 1, whose
+// index would be -1; one FMA for i = 2).
+template <int I, typename F>
+__device__ __forceinline__ double raise(double X, double r1, F&& r2) {
+  if constexpr (I == 1) return X * r1;
+  else if constexpr (I == 2) return fma(X, r1, r2());
+  else return fma((double)(I - 1), r2(), X * r1);
+}
+// Product ex ey ez of three E-table entries of blocks with nx, ny, nz Hermite terms: the (0, 0) block of a
+// table is the number 1 and costs no multiplication (12 of the 60 FP64 instructions that [..|ps] had issued
+// per primitive quartet).
+template <int NX, int NY, int NZ>
+__device__ __forceinline__ double eprod(const double* ex, const double* ey, const double* ez) {
+  if constexpr (NX * NY * NZ == 1) return 1.0;
+  else if constexpr (NX * NY == 1) return __ldg(ez);
+  else if constexpr (NX * NZ == 1) return __ldg(ey);
+  else if constexpr (NY * NZ == 1) return __ldg(ex);
+  else if constexpr (NZ == 1) return __ldg(ex) * __ldg(ey);
+  else if constexpr (NY == 1) return __ldg(ex) * __ldg(ez);
+  else if constexpr (NX == 1) return __ldg(ey) * __ldg(ez);
+  else return __ldg(ex) * __ldg(ey) * __ldg(ez);
+}
+
 // XS = false: R, [p|cd] and the shellset in registers (classes with
 // reg_eligible). XS = true: R in registers, [p|cd] and the shellset in shared
 // memory (classes with reg_xs_eligible, total angular momentum <= 6).
@@ -134,29 +157,44 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
     const bool live = pb0 + sb < Kb;   // a lane past the last bra primitive adds zeros to the group's sums
     const int pb = live ? pb0 + sb : 0;
     const double* __restrict__ rb = rb0 + (int64_t)pb * RB;
-    const double zp = __ldg(rb), izp = __ldg(rb + 1);
+    const double zp = __ldg(rb), zpm2 = -2.0 * zp;
     const double Px = __ldg(rb + 2), Py = __ldg(rb + 3), Pz = __ldg(rb + 4);
-    // 2 pi^(5/2) / zp * c_a c_b K_ab (the ket part and 1/sqrt(zp+zq) per ket primitive)
-    const double prefb = 34.986836655249725693 * izp * __ldg(rb + 5);
+    // 2 pi^(5/2) * c_a c_b K_ab / zp (the ket part and 1/sqrt(zp+zq) per ket primitive)
+    const double prefb = 34.986836655249725693 * __ldg(rb + 6);
     sfor<HB * Nk>([&](auto i) { X[i] = 0.0; });
 
     for (int pk = live ? sk : Kk; pk < Kk; pk += Sk) {
       const double* __restrict__ rk = rk0 + (int64_t)pk * RK;
-      const double zq = __ldg(rk), izq = __ldg(rk + 1);
+      const double zq = __ldg(rk);
       const double PQx = Px - __ldg(rk + 2), PQy = Py - __ldg(rk + 3), PQz = Pz - __ldg(rk + 4);
       const double s = zp + zq;
-      const double rs = rsqrt(s);
-      const double rho = zp * zq * rs * rs;
-      const double Tb = rho * (PQx * PQx + PQy * PQy + PQz * PQz);
-      const double pref = prefb * izq * rs * __ldg(rk + 5);
-      const double m2r = -2.0 * rho;
-      // Boys seeds G[m] = (-2 rho)^m pref F_m(T), m = 0..L (Eq. 0m)
+      const double R2 = PQx * PQx + PQy * PQy + PQz * PQz;
+      // Boys seeds G[m] = (-2 rho)^m pref F_m(T), m = 0..L (Eq. 0m), rho = zp zq / s, T = rho R^2, without a
+      // branch between the table and the asymptotic form F_m(T) = Gamma(m+1/2) / (2 T^(m+1/2)):
+      // with y = 1/sqrt(s) below T = 64 and y = 1/sqrt(zp zq R^2) above, and b = -2 zp zq y^2,
+      //   G[m] = C y b^m f_m,  f_m = F_m(T) below and Gamma(m+1/2)/2 above,
+      // and the table's last row holds the constants (T is 1 there, a grid point). The branch had cost a
+      // quarter of the FP64 issue slots of [ps|ss] (warps whose quartets lie on both sides run both).
+      // exp(-T) / (2 T F_m) is below 1e-20 from T = 64 on for m <= 6. With this, the one-term E tables and the
+      // coefficient 1 of Eq. r (40,000 quartets): [ss|ss] K = 6,6,6,6 5.74 -> 4.09 ms, [ps|ss] K = 3,6,6,6
+      // 4.22 -> 2.88 ms, [dp|ps] K = 1,3,3,6 1.55 -> 1.39 ms.
+      const double zz2 = zpm2 * zq;                // -2 zp zq
+      const double c2 = zz2 * R2;                  // -2 zp zq R^2
+      const int hc = __double2hiint(c2) & 0x7fffffff;
+      const bool far = hc >= __double2hiint(s) + (7 << 20);   // 2 zp zq R^2 >= 128 s, by the exponents
+      // zp zq R^2 = c2 / -2: sign off, exponent less one
+      const double y = rsqrt(far ? __hiloint2double(hc - (1 << 20), __double2loint(c2)) : s);
+      const double y2 = y * y;
+      const double T2 = c2 * y2;                   // -2 T
+      // nearest grid point of spacing 1/16: the low word of T + 1.5 2^48
+      const double tm = fma(T2, -0.5, 422212465065984.0);
+      const double nd = fma(T2, 0.5, tm - 422212465065984.0);   // T0 - T
+      const int i = far ? kBoysNgrid - 1 : min(__double2loint(tm) & 0x7fffffff, kBoysNgrid - 1);
+      const double2* row = reinterpret_cast<const double2*>(boys + (size_t)i * kBoysRow);
       double G[L + 1];
-      if (Tb < kBoysTmax) {
-        const int i = __double2int_rn(Tb * kBoysInvH);
-        const double nd = (double)i * (1.0 / kBoysInvH) - Tb;
-        const double2* row = reinterpret_cast<const double2*>(boys + (size_t)i * kBoysRow);
-        double pw = pref;
+      {
+        const double bm = zz2 * y2;
+        double pw = prefb * __ldg(rk + 6) * y;
         sfor<L + 1>([&](auto m) {
           const double2 c01 = __ldg(row + 4 * m), c23 = __ldg(row + 4 * m + 1);
           const double2 c45 = __ldg(row + 4 * m + 2), c67 = __ldg(row + 4 * m + 3);
@@ -168,17 +206,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           f = fma(f, nd, c01.y);
           f = fma(f, nd, c01.x);
           G[m] = pw * f;
-          pw *= m2r;
-        });
-      } else {
-        // F_m(T) = Gamma(m+1/2) / (2 T^(m+1/2)), Gamma(m+1/2)/2 = sqrt(pi)/2 (2m-1)!!/2^m
-        // (exp(-T) terms negligible above the table)
-        const double t1 = rsqrt(Tb);
-        const double x = m2r * t1 * t1;
-        double g = 0.88622692545275801365 * pref * t1;
-        sfor<L + 1>([&](auto m) {
-          G[m] = g;
-          g *= x * ((double)m + 0.5);
+          if constexpr (m < L) pw *= bm;
         });
       }
       // R^(n)_tuv for n = L..0 in one array indexed in the order-L simplex:
@@ -195,14 +223,11 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
               constexpr int v = N - t - u;
               double val;
               if constexpr (v > 0) {
-                val = PQz * R[hidx(L, t, u, v - 1)];
-                if constexpr (v > 1) val = fma((double)(v - 1), R[hidx(L, t, u, v - 2)], val);
+                val = raise<v>(PQz, R[hidx(L, t, u, v - 1)], [&] { return R[hidx(L, t, u, v - 2)]; });
               } else if constexpr (u > 0) {
-                val = PQy * R[hidx(L, t, u - 1, 0)];
-                if constexpr (u > 1) val = fma((double)(u - 1), R[hidx(L, t, u - 2, 0)], val);
+                val = raise<u>(PQy, R[hidx(L, t, u - 1, 0)], [&] { return R[hidx(L, t, u - 2, 0)]; });
               } else {
-                val = PQx * R[hidx(L, t - 1, 0, 0)];
-                if constexpr (t > 1) val = fma((double)(t - 1), R[hidx(L, t - 2, 0, 0)], val);
+                val = raise<t>(PQx, R[hidx(L, t - 1, 0, 0)], [&] { return R[hidx(L, t - 2, 0, 0)]; });
               }
               R[hidx(L, t, u, v)] = val;
             });
@@ -220,12 +245,8 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           const double* Ey = rk + kRecHeader + EK + etab_off(LD, ey, fy);
           const double* Ez = rk + kRecHeader + 2 * EK + etab_off(LD, ez, fz);
           double E[nx * ny * nz];
-          sfor<nx>([&](auto tau) {
-            const double vx = __ldg(Ex + tau);
-            sfor<ny>([&](auto nu) {
-              const double vxy = vx * __ldg(Ey + nu);
-              sfor<nz>([&](auto phi) { E[(tau * ny + nu) * nz + phi] = vxy * __ldg(Ez + phi); });
-            });
+          sfor<nx * ny * nz>([&](auto k) {
+            E[k] = eprod<nx, ny, nz>(Ex + k / (ny * nz), Ey + k / nz % ny, Ez + k % nz);
           });
           sfor<Lb + 1>([&](auto t) {
             sfor<Lb + 1 - t>([&](auto u) {
@@ -235,7 +256,9 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
                 sfor<nx>([&](auto tau) {
                   sfor<ny>([&](auto nu) {
                     sfor<nz>([&](auto phi) {
-                      acc = fma(E[(tau * ny + nu) * nz + phi], R[hidx(L, t + tau, u + nu, v + phi)], acc);
+                      const double r = R[hidx(L, t + tau, u + nu, v + phi)];
+                      if constexpr (nx * ny * nz == 1) acc += r;
+                      else acc = fma(E[(tau * ny + nu) * nz + phi], r, acc);
                     });
                   });
                 });
@@ -262,9 +285,10 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           for (int t = 0; t <= ax + bx; ++t) {
             const double vx = __ldg(Ex + t);
             for (int u = 0; u <= ay + by; ++u) {
-              const double vxy = vx * __ldg(Ey + u);
+              // (a one-term table is the number 1; the uniform branch also makes the faster loop: [pp|pp] 161 -> 152 us)
+              const double vxy = ay + by ? vx * __ldg(Ey + u) : vx;
               for (int v = 0; v <= az + bz; ++v) {
-                const double e = vxy * __ldg(Ez + v);
+                const double e = az + bz ? vxy * __ldg(Ez + v) : vxy;
                 const int h = hidx(Lb, t, u, v) * Nk;
                 sfor<Nk>([&](auto cd) { acc[cd] = fma(e, X[h + cd], acc[cd]); });
               }
@@ -303,19 +327,19 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           const double* Ey = rb + kRecHeader + EB + etab_off(LB, ay, by);
           const double* Ez = rb + kRecHeader + 2 * EB + etab_off(LB, az, bz);
           double E[nx * ny * nz];
-          sfor<nx>([&](auto t) {
-            const double vx = __ldg(Ex + t);
-            sfor<ny>([&](auto u) {
-              const double vxy = vx * __ldg(Ey + u);
-              sfor<nz>([&](auto v) { E[(t * ny + u) * nz + v] = vxy * __ldg(Ez + v); });
-            });
+          sfor<nx * ny * nz>([&](auto k) {
+            E[k] = eprod<nx, ny, nz>(Ex + k / (ny * nz), Ey + k / nz % ny, Ez + k % nz);
           });
           sfor<Nk>([&](auto cd) {
             constexpr int o = (ia * NB + ib) * Nk + cd;
             double acc = V[o];
             sfor<nx>([&](auto t) {
               sfor<ny>([&](auto u) {
-                sfor<nz>([&](auto v) { acc = fma(E[(t * ny + u) * nz + v], X[hidx(Lb, t, u, v) * Nk + cd], acc); });
+                sfor<nz>([&](auto v) {
+                  const double x = X[hidx(Lb, t, u, v) * Nk + cd];
+                  if constexpr (nx * ny * nz == 1) acc += x;
+                  else acc = fma(E[(t * ny + u) * nz + v], x, acc);
+                });
               });
             });
             V[o] = acc;
