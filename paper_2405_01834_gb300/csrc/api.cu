@@ -40,6 +40,7 @@ struct mdx_ctx {
   int device = 0;
   std::string last_error;
   double* d_boys = nullptr;
+  double* d_rys = nullptr;                // Rys nodes and weights, uploaded when a class first needs them
   uint32_t* d_rprog = nullptr;
   int32_t* d_rprog_off = nullptr;
   int* d_err = nullptr;
@@ -145,6 +146,23 @@ mdx_status get_plan(mdx_ctx* c, const ClassKey& k, Plan** out, cudaStream_t s) {
   if (st != MDX_OK) { if (p->dev_blob) cudaFree(p->dev_blob); return st; }
   *out = p.get();
   c->plans[k] = std::move(p);
+  return MDX_OK;
+}
+
+mdx_status need_rys_table(mdx_ctx* c) {
+  if (c->d_rys) return MDX_OK;
+  const std::vector<double>& tab = rys_table();
+  double* p = nullptr;
+  if (cudaMalloc((void**)&p, tab.size() * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(c, MDX_ENOMEM, "Rys table allocation failed");
+  }
+  const cudaError_t e = cudaMemcpy(p, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return cuda_fail(c, e, "Rys table upload");
+  }
+  c->d_rys = p;
   return MDX_OK;
 }
 
@@ -450,6 +468,13 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
     Plan* splan = nullptr;
     int grid = 0;
     double fma = plan->exec_fma;
+    if (!sph && plan->d.rys) {
+      if ((st = need_rys_table(c)) != MDX_OK) return st;
+      cudaError_t e = rys_grid(plan->d, cnt, &grid);
+      if (e != cudaSuccess) return cuda_fail(c, e, "Rys launch shape");
+      xg_total = std::max<int64_t>(xg_total, (int64_t)grid * plan->d.ry_table);
+      fma = plan->rys_fma;
+    }
     ClassKey ks = kv.first;
     ks.store = 2;
     // the solid-harmonic team kernel: every class without a register kernel, and those the autotuner moved
@@ -505,6 +530,15 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
       cudaGetLastError();
       return fail(c, MDX_ENOMEM, "record allocation failed");
     }
+  }
+  if (!sph && xg_total > 0) {   // the global axis tables of the largest Rys classes
+    if (call_ws) {
+      if ((st = ensure(c, "call_rys", (size_t)xg_total, &B->xg, s)) != MDX_OK) return st;
+    } else if (cudaMalloc(&B->xg, xg_total * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(c, MDX_ENOMEM, "Rys table area allocation failed");
+    }
+    B->nxg = xg_total;
   }
   if (sph) {
     if ((st = dev_upload(c, cqoff, &B->cqoff, s)) != MDX_OK) return st;
@@ -562,7 +596,21 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
       ++nl;
       continue;
     }
+    if (!B->sph && r.plan->d.ry_stash) {   // one area of axis tables for all of them: one stream
+      a.rys = c->d_rys;
+      a.sph_scratch = B->xg;
+      fan.load[0] += B->order[i].first;
+      e = launch_rys(a, r.grid, s);
+      ++nl;
+      continue;
+    }
     const cudaStream_t rs = fan.stream(fan.pick(B->order[i].first));
+    if (!B->sph && r.plan->d.rys) {
+      a.rys = c->d_rys;
+      e = launch_rys(a, r.grid, rs);
+      ++nl;
+      continue;
+    }
     if (B->sph) {              // Cartesian shellsets, then the index-by-index transform
       a.qout = B->cqoff + r.begin;
       a.out = B->cart;
@@ -757,6 +805,7 @@ void mdx_destroy(mdx_ctx* c) {
   for (auto& p : c->retired) if (p->dev_blob) cudaFree(p->dev_blob);
   for (auto& kv : c->bufs) if (kv.second.p) cudaFree(kv.second.p);
   cudaFree(c->d_boys);
+  cudaFree(c->d_rys);
   cudaFree(c->d_rprog);
   cudaFree(c->d_rprog_off);
   cudaFree(c->d_err);
@@ -1229,6 +1278,30 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
     if (reg_eligible(rk.la, rk.lb, rk.lc, rk.ld) || reg_xs_eligible(rk.la, rk.lb, rk.lc, rk.ld))
       cands.push_back(PlanConfig{0, 200 * 1024, 96 * 1024, 2});
     float best_ms = 1e30f;
+    if (r.plan->d.rys) {   // a class of the Rys kernel keeps it unless a team shape is faster
+      QuartetLaunch a{};
+      a.plan = r.plan->d;
+      a.nq = std::min(r.count, max_trial);
+      a.qpairs = b->qp + r.begin;
+      a.qout = b->qoff + r.begin;
+      a.pair_rec = b->pair_rec;
+      a.recs = b->recs;
+      a.recs_signed = b->recs_s;
+      a.rys = c->d_rys;
+      a.sph_scratch = b->xg;
+      a.out = out;
+      a.err = c->d_err;
+      for (int rep = 0; rep < 2; ++rep) {
+        cudaEventRecord(e0, s);
+        e = launch_rys(a, (int)std::min<int64_t>(r.grid, a.nq), s);
+        cudaEventRecord(e1, s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e != cudaSuccess) { cudaEventDestroy(e0); cudaEventDestroy(e1); return cuda_fail(c, e, "autotune"); }
+        float t = 0;
+        cudaEventElapsedTime(&t, e0, e1);
+        best_ms = std::min(best_ms, t);
+      }
+    }
     PlanConfig best{};
     std::unique_ptr<Plan> best_plan;
     std::vector<std::pair<int, int>> seen;   // (T, team_doubles, ngroups) signature of built plans
@@ -1277,7 +1350,8 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
     }
     if (!best_plan) continue;
     c->tuned[r.key] = best;
-    b->exec_fma += (best_plan->exec_fma - r.plan->exec_fma) * (double)r.count;   // the shape it runs now
+    b->exec_fma += (best_plan->exec_fma - (r.plan->d.rys ? r.plan->rys_fma : r.plan->exec_fma)) *
+                   (double)r.count;   // the shape it runs now
     auto it = c->plans.find(r.key);
     if (it != c->plans.end()) c->retired.push_back(std::move(it->second));
     r.plan = best_plan.get();

@@ -1476,6 +1476,8 @@ cudaError_t kernel_attributes_init() {
     e = cudaMemcpyToSymbol(c_top, top, sizeof(top));
     if (e != cudaSuccess) return e;
   }
+  e = rys_attributes_init();
+  if (e != cudaSuccess) return e;
   const int maxshm = 227 * 1024;
   e = cudaFuncSetAttribute(k_quartets<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxshm);
   if (e != cudaSuccess) return e;

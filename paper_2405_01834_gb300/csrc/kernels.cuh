@@ -40,6 +40,7 @@ struct QuartetLaunch {
   const double* recs;
   const double* recs_signed;
   const double* boys;
+  const double* rys;         // Rys nodes and weights (rys_table); null where no launch needs them
   const uint32_t* rprog;     // R-level programs (one word per Hermite entry, build_rlevel_programs)
   const int32_t* rprog_off;  // start of each total order N in rprog
   double* out;
@@ -103,6 +104,11 @@ cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s);
 // grid * teams_per_cta * xg_doubles doubles.
 cudaError_t sph_grid(const PlanDev& P, int64_t nq, int* grid);
 cudaError_t launch_quartets_sph(const QuartetLaunch& a, int grid, cudaStream_t s);
+// Rys kernel (plan.rys, store epilogue): rys_grid gives the grid for nq quartets; with plan.ry_stash, a.sph_scratch
+// must hold grid * ry_table doubles.
+cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid);
+cudaError_t launch_rys(const QuartetLaunch& a, int grid, cudaStream_t s);
+cudaError_t rys_attributes_init();
 // Writes zeros over n output ranges given as (offset, doubles) pairs (screened-out shellsets).
 cudaError_t launch_zero_ranges(const int64_t* ranges, int64_t n, double* out, cudaStream_t s);
 // Gradient epilogue over shellsets already in memory (V + q N_b N_k for quartet q of launch a).

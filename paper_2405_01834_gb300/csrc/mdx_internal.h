@@ -27,6 +27,15 @@ constexpr int kBoysNgrid = 1601 + 1;                // T0 = 0 .. 100, and a last
 // (row-major) in long double by downward recursion (see boys_table.cpp).
 std::vector<double> build_boys_table();
 
+// ----------------------------------------------------------------- Rys quadrature
+constexpr int kRysMax = 2 * kLmax + 1;     // nodes for total angular momentum 4 l_max
+constexpr int kRysTerms = 13;              // polynomial coefficients per interval
+constexpr int kRysIntervals = 100;         // unit intervals of T; the limit form above
+// Rule of n nodes at rys_offset(n): per interval i (T - (i + 1/2) in [-1/2, 1/2]) and power k the n nodes t_r^2
+// and the n weights; then the n nodes X_r and n half weights W_r / 2 of the limit form.
+constexpr int64_t rys_offset(int n) { return (int64_t)n * (n - 1) * (kRysTerms * kRysIntervals + 1); }
+const std::vector<double>& rys_table();    // rys_table.cpp; built on first use
+
 // ----------------------------------------------------------------- records
 // Primitive-pair record: header of kRecHeader doubles, then the three per-axis
 // E tables (x, y, z). Header: [0] zeta_p, [1] 1/zeta_p, [2..4] P, [5] prefactor
@@ -171,6 +180,11 @@ struct PlanDev {
   // lower Hermite term of its Cartesian expansion cancels), so the ket steps form only the rows |p| = l_a
   // and the bra step is OUT[m] = (2 zeta)^-l_a sum_a C_ma [a|cd] over those rows
   int32_t top_only;
+  // Rys kernel (store launches of one primitive quartet; rys_kernel.cu): number of nodes, 0 if the class does
+  // not take it; threads per block; shared memory (doubles) and its regions; ket indices c per table chunk;
+  // ry_stash: the tables live in a global area of ry_table doubles per block
+  int32_t rys, ry_threads, ry_doubles, ry_h, ry_N, ry_T, ry_idx, ry_cw, ry_stash;
+  int64_t ry_table;
   float cost_k, cost_b;                  // a team's chain (clocks, roughly) per primitive quartet and per bra transform
   int64_t xg_doubles;                    // staging per team: Xg [Nk][hbp] then Yg [nc_c * nsd][hbp]
   const Group* groups;
@@ -190,6 +204,7 @@ struct Plan {
   std::vector<uint16_t> colmap;
   std::vector<uint16_t> colinv;
   double exec_fma = 0;     // FMAs executed per primitive-quartet pass (for reports)
+  double rys_fma = 0;      // FP64 instructions of the Rys kernel per shellset (d.rys)
   void* dev_blob = nullptr;
 };
 
@@ -202,9 +217,10 @@ struct PlanConfig {
   int rcache = -1;           // cached R tables of contracted multi-group classes: -1 where they fit without
                              // costing occupancy, 0 never, 1 wherever they fit
   int pack_zpairs = 1;       // small ket z-pairs share column groups (0: one group or more per z-pair)
+  int rys = -1;              // Rys kernel for shellset output: -1 where it executes less, 0 never
   bool operator==(const PlanConfig& o) const {
     return T == o.T && budget == o.budget && single_max == o.single_max && variant == o.variant &&
-           rcache == o.rcache && pack_zpairs == o.pack_zpairs;
+           rcache == o.rcache && rys == o.rys && pack_zpairs == o.pack_zpairs;
   }
 };
 

@@ -175,7 +175,9 @@ extern "C" mdx_status mdx_eri4_noalloc(const mdx_basis* basis, const int32_t* qu
     if (it == g_plans.end()) {
       std::unique_ptr<Plan> p(new Plan());
       std::string err;
-      if (!build_plan(kv.first, PlanConfig{}, *p, err)) return MDX_EUNSUPPORTED;
+      PlanConfig cfg{};
+      cfg.rys = 0;   // its tables have no place in the fixed scratch
+      if (!build_plan(kv.first, cfg, *p, err)) return MDX_EUNSUPPORTED;
       it = g_plans.emplace(kv.first, std::move(p)).first;
     }
     const int64_t b = (int64_t)qp_sorted.size();

@@ -245,6 +245,49 @@ bool validate_plan(const Plan& plan, std::string& err) {
 
 }  // namespace
 
+// Rys kernel of an uncontracted class (rys_kernel.cu): its shared-memory layout, block size and FP64
+// instruction count, where it executes fewer than the step programs.
+static void plan_rys(Plan& plan) {
+  PlanDev& P = plan.d;
+  const int n = P.L / 2 + 1;
+  const int nab1 = (P.la + 1) * (P.lb + 1), ncd1 = (P.lc + 1) * (P.ld + 1);
+  auto terms = [](int l1, int l2) {   // Hermite terms over the one-axis index pairs
+    double t = 0;
+    for (int x = 0; x <= l1; ++x)
+      for (int y = 0; y <= l2; ++y) t += x + y + 1;
+    return t;
+  };
+  plan.rys_fma = 2.0 * n * P.Nb * P.Nk + 3.0 * n * (terms(P.la, P.lb) * ncd1 + (P.Lb + 1) * terms(P.lc, P.ld)) +
+                 3.0 * n * 2.0 * P.L + 2.0 * n * kRysTerms;
+  // Both are bound by the FP64 pipe, so the count decides. Measured (team kernel -> this one, same grids):
+  // [61|00] 627 -> 432 us, [22|22] 2.08 -> 1.42 ms, [ff|ff] 4.02 -> 2.40 ms, [ii|ii] 27.5 -> 14.8 ms, 3-center
+  // [6|10] 476 -> 378 us, [3|33] 6.48 -> 1.62 ms, [6|66] 11.6 -> 4.63 ms; no class of L >= 7 was slower.
+  if (n > kRysMax || plan.rys_fma > 0.97 * plan.exec_fma) return;
+  const int fixed = P.recb + P.reck + 2 * n + 3 * (P.L + 1) * n + ((P.Nb + P.Nk + nab1 + ncd1 + 1) / 2 + 1);
+  auto doubles = [&](int cw, int rows) {
+    return fixed + 3 * (P.Lb + 1) * n * cw * (P.ld + 1) + 3 * rows * n * ncd1;
+  };
+  const int cap = 225 * 1024 / 8;
+  P.ry_stash = doubles(P.lc + 1, nab1) > cap && doubles(1, nab1) > cap;
+  const int rows = P.ry_stash ? P.lb + 1 : nab1;
+  // tables that stay in shared memory: all ket indices in one chunk where that fits; rows of a global table: as
+  // many as leave room for two blocks per SM
+  P.ry_cw = P.lc + 1;
+  while (P.ry_cw > 1 && doubles(P.ry_cw, rows) > (P.ry_stash ? cap / 2 : cap)) --P.ry_cw;
+  if (doubles(P.ry_cw, rows) > cap) return;
+  P.ry_h = P.recb + P.reck;
+  P.ry_N = P.ry_h + 2 * n + 3 * (P.L + 1) * n;
+  P.ry_T = P.ry_N + 3 * (P.Lb + 1) * n * P.ry_cw * (P.ld + 1);
+  P.ry_idx = P.ry_T + 3 * rows * n * ncd1;
+  P.ry_doubles = doubles(P.ry_cw, rows);
+  P.ry_table = P.ry_stash ? (int64_t)3 * nab1 * n * ncd1 : 0;
+  // enough threads that the blocks an SM holds are 16 warps together
+  const int blocks = std::max(1, (int)(228L * 1024 / (P.ry_doubles * 8 + 1024)));
+  P.ry_threads = 64;
+  while (P.ry_threads < 512 && P.ry_threads * blocks < 512) P.ry_threads *= 2;
+  P.rys = n;
+}
+
 void build_rlevel_programs(std::vector<uint32_t>& prog, std::vector<int32_t>& off) {
   prog.clear();
   off.clear();
@@ -689,6 +732,8 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
         p2.exec_fma + 2.0 * r_alt < 0.9 * (plan.exec_fma + 2.0 * r_cur))
       plan = std::move(p2);
   }
+  if (key.store == 1 && key.Kb * key.Kk == 1 && !P.reg && cfg.variant == 0 && cfg.T == 0 && cfg.rys != 0)
+    plan_rys(plan);
   return true;
 }
 
