@@ -284,6 +284,87 @@ __device__ void compute_R(const QuartetLaunch& a, double* ws, int tl, unsigned m
   }
 }
 
+// The R tables of `m` primitive quartets of one quartet at once: table j (j < m) is that of bra primitive pair
+// pb(i) = b0 + (i / nk) bs and ket pair pk(i) = k0 + (i % nk) ks, i = first + j, written to tab + j rstride.
+// Per primitive quartet a team pays a chain of L + 4 barriers, most of them with a handful of working lanes (Boys
+// seeds: L + 1; the first levels: 3, 9, 19 entries), and the warp that forms T and the prefactor for a single
+// primitive pays their 35 FP64 instructions for one; a batch pays both once. Measured (team kernel, store): [dd|dd]
+// K = 81 9.70 -> 8.51 ms for 3,600 quartets, [dd|dp] 5.24 -> 4.30, [fp|pp] K = 27 2.37 -> 1.91 ms for 10,000,
+// [hh|sp] K = 18 1.23 -> 0.99 ms; 6-atom one-shot call 7.7 -> 6.7 ms.
+// work: m kb_work(L) doubles. Ends with a barrier.
+struct RBatch {
+  int b0, bs, k0, ks, nk;
+};
+template <bool CTA>
+__device__ void compute_R_batch(const QuartetLaunch& a, int64_t bra0, int64_t ket0, const RBatch bt, int first, int m,
+                                double* tab, double* work, int tl, unsigned mask) {
+  const PlanDev& P = a.plan;
+  const int T = P.T, L = P.L, rstride = P.rstride, n1 = d_tet(L);
+  double* odd = work;                 // [j][n1]: levels n odd
+  double* hdr = work + m * n1;        // [j][6]
+  double* G = hdr + 6 * m;            // [j][L + 1]
+  for (int j = tl; j < m; j += T) {
+    const int i = first + j, ib = i / bt.nk, pb = bt.b0 + ib * bt.bs, pk = bt.k0 + (i - ib * bt.nk) * bt.ks;
+    const double* rb = a.recs + bra0 + (int64_t)pb * P.recb;
+    const double* rk = a.recs_signed + ket0 + (int64_t)pk * P.reck;
+    const double zp = __ldg(rb), zq = __ldg(rk);
+    const double X = __ldg(rb + 2) - __ldg(rk + 2), Y = __ldg(rb + 3) - __ldg(rk + 3), Z = __ldg(rb + 4) - __ldg(rk + 4);
+    const double rs = rsqrt(zp + zq);
+    const double rho = zp * zq * rs * rs;
+    double* h = hdr + 6 * j;
+    h[0] = X; h[1] = Y; h[2] = Z;
+    h[3] = rho * (X * X + Y * Y + Z * Z);
+    h[4] = 34.986836655249725693 * __ldg(rb + 6) * __ldg(rk + 6) * rs;
+    h[5] = -2.0 * rho;
+  }
+  team_sync<CTA>(mask);
+  const float inv1 = 1.0f / (float)(L + 1);
+  for (int e = tl; e < m * (L + 1); e += T) {
+    const int j = (int)(((float)e + 0.5f) * inv1), o = e - j * (L + 1);
+    const double* h = hdr + 6 * j;
+    const double Tb = h[3];
+    double f, b = h[5];
+    if (Tb < kBoysTmax) {
+      const int i = __double2int_rn(Tb * kBoysInvH);
+      const double nd = (double)i * (1.0 / kBoysInvH) - Tb;
+      const double2* c = reinterpret_cast<const double2*>(a.boys + (size_t)i * kBoysRow + o * kBoysTerms);
+      const double2 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2), c67 = __ldg(c + 3);
+      f = fma(c67.y, nd, c67.x);
+      f = fma(f, nd, c45.y);
+      f = fma(f, nd, c45.x);
+      f = fma(f, nd, c23.y);
+      f = fma(f, nd, c23.x);
+      f = fma(f, nd, c01.y);
+      f = fma(f, nd, c01.x);
+    } else {
+      const double y = rsqrt(Tb);   // F_m(T) = Gamma(m+1/2) / (2 T^(m+1/2))
+      b *= y * y;
+      f = c_gh[o] * y;
+    }
+    G[e] = f * h[4] * ipow(b, o);
+    if (o == L) ((L & 1) ? odd + j * n1 : tab + j * rstride)[0] = G[e];
+  }
+  team_sync<CTA>(mask);
+  for (int n = L - 1; n >= 0; --n) {
+    const int N = L - n;
+    double* dst = (n & 1) ? odd : tab;
+    const double* src = (n & 1) ? tab : odd;
+    const int sd = (n & 1) ? n1 : rstride, ss = (n & 1) ? rstride : n1;
+    const uint32_t* prog = a.rprog + a.rprog_off[N];
+    const int cnt = d_tet(N + 1);
+    const float inv = 1.0f / (float)cnt;
+    for (int i = tl; i < m * cnt; i += T) {
+      const int j = (int)(((float)i + 0.5f) * inv), e = i - j * cnt;   // i / cnt: i < 2^17, so exact
+      const uint32_t w = __ldg(prog + e);
+      const double* sj = src + j * ss;
+      double val = hdr[6 * j + ((w >> 24) & 3)] * sj[w & 0xfff];
+      val = fma(__ldg(g_dint + (w >> 26)), sj[(w >> 12) & 0xfff], val);
+      dst[j * sd + e] = e == 0 ? G[j * (L + 1) + n] : val;
+    }
+    team_sync<CTA>(mask);
+  }
+}
+
 // Two dot products side by side, operands loaded one term ahead of the FMAs
 // that consume them (shared-memory latency overlaps the FP64 pipe).
 __device__ __forceinline__ void dual_dot(const double* __restrict__ c0, const double* __restrict__ x0, int st0, int n0,
@@ -310,8 +391,11 @@ __device__ __forceinline__ void dual_dot(const double* __restrict__ c0, const do
 // chains hide the FP64 pipe latency. Entries are sorted by length, so the
 // two usually have the same n. The next pair of entries is fetched while the
 // current pair is computed.
+// dsrc, dcoef: shifts of the sources and of the coefficients (the R table and the record of a batch slot).
 __device__ __forceinline__ void run_step(const StepEntry* __restrict__ prog, int n, double* ws, int tl, int T,
-                                         bool acc) {
+                                         bool acc, int dsrc = 0, int dcoef = 0) {
+  const double* wx = ws + dsrc;
+  const double* wc = ws + dcoef;
   int e = tl;
   StepEntry p0{}, p1{};
   if (e + T < n) { p0 = prog[e]; p1 = prog[e + T]; }
@@ -320,14 +404,14 @@ __device__ __forceinline__ void run_step(const StepEntry* __restrict__ prog, int
     if (e + 3 * T < n) { p0 = prog[e + 2 * T]; p1 = prog[e + 3 * T]; }
     double v0 = acc ? ws[s0.out] : 0.0;
     double v1 = acc ? ws[s1.out] : 0.0;
-    dual_dot(ws + s0.coef, ws + s0.src, s0.stride, s0.n, ws + s1.coef, ws + s1.src, s1.stride, s1.n, v0, v1);
+    dual_dot(wc + s0.coef, wx + s0.src, s0.stride, s0.n, wc + s1.coef, wx + s1.src, s1.stride, s1.n, v0, v1);
     ws[s0.out] = v0;
     ws[s1.out] = v1;
   }
   if (e < n) {
     const StepEntry s = prog[e];
-    const double* c = ws + s.coef;
-    const double* x = ws + s.src;
+    const double* c = wc + s.coef;
+    const double* x = wx + s.src;
     const int st = s.stride;
     double v = acc ? ws[s.out] : 0.0;
     for (int k = 0; k < s.n; ++k) v = fma(c[k * st], x[k * st], v);
@@ -661,9 +745,9 @@ __device__ __forceinline__ void load_cached_R(const PlanDev& P, double* ws, int 
   for (int e = tl; e < nR; e += P.T) ws[P.o_R0 + e] = src[e];
 }
 
-// The R tables of the primitive quartets of bra primitives pb0 <= pb < pb1 of
-// q, computed once and kept in the workspace region o_Rc, table
-// (pb - pb0) Kk + pk (plans with cache_R == 2: every primitive quartet, filled
+// The R tables of the team's primitive quartets of bra primitives pb0 <= pb < pb1
+// of q, computed once and kept in the workspace region o_Rc, one after another
+// in the order of its loops (plans with cache_R == 2: every primitive quartet, filled
 // once per quartet; cache_R == 3, solid-harmonic plans: those of one bra
 // primitive, filled per bra primitive). Contracted classes of several column
 // groups would otherwise compute each R once per group.
@@ -671,17 +755,11 @@ template <bool CTA>
 __device__ __forceinline__ void fill_R_cache(const QuartetLaunch& a, double* ws, int64_t bra0, int64_t ket0, int pb0,
                                              int pb1, int tl, unsigned mask, PrimPart part = PrimPart{0, 1, 0, 1}) {
   const PlanDev& P = a.plan;
-  const int nR = d_tet(P.L + 1);
-  for (int pb = pb0 + part.b; pb < pb1; pb += part.nb)
-    for (int pk = part.k; pk < P.Kk; pk += part.nk) {
-      load_record(ws + P.o_recb, a.recs + bra0 + (int64_t)pb * P.recb, P.recb, tl, P.T);
-      load_record(ws + P.o_reck, a.recs_signed + ket0 + (int64_t)pk * P.reck, P.reck, tl, P.T);
-      team_sync<CTA>(mask);   // also orders the previous table's copy before compute_R rewrites R0
-      compute_R<CTA>(a, ws, tl, mask);
-      double* dst = ws + P.o_Rc + (int64_t)((pb - pb0) * P.Kk + pk) * P.rstride;
-      for (int e = tl; e < nR; e += P.T) dst[e] = ws[P.o_R0 + e];
-    }
-  team_sync<CTA>(mask);
+  const int nb = (pb1 - pb0 - part.b + part.nb - 1) / part.nb, nk = (P.Kk - part.k + part.nk - 1) / part.nk;
+  const RBatch bt{pb0 + part.b, part.nb, part.k, part.nk, nk};
+  for (int i = 0; i < nb * nk; i += P.kb_m)
+    compute_R_batch<CTA>(a, bra0, ket0, bt, i, min(P.kb_m, nb * nk - i), ws + P.o_Rc + (int64_t)i * P.rstride,
+                         ws + P.o_KS, tl, mask);
 }
 
 // The work of one team on one shell quartet q (all groups, all primitives,
@@ -716,13 +794,38 @@ __device__ __forceinline__ void quartet_body(const QuartetLaunch& a, double* ws,
   for (int g = 0; g < P.ngroups; ++g) {
     const Group grp = P.groups[g];
     const int ncols = grp.ncols;
+    int icache = 0;   // table of the cache (cache_R == 2), in the order of these loops
     for (int pb = part.b; pb < Kb; pb += part.nb) {
       const bool last_b = pb + part.nb >= Kb;
       if (P.cache_R != 1) load_record(ws + P.o_recb, a.recs + bra0 + (int64_t)pb * P.recb, P.recb, tl, T);
-      for (int pk = part.k; pk < Kk; pk += part.nk) {
+      if (P.cache_R == 0 && P.kb_m > 0) {
+        // batches of ket primitives: their R tables together, then the steps of each from its slot
+        const int nk = (Kk - part.k + part.nk - 1) / part.nk;
+        for (int i0 = 0; i0 < nk; i0 += P.kb_m) {
+          const int m = min(P.kb_m, nk - i0);
+          // (one batch holds all the ket records: they stay from one bra primitive to the next)
+          if (pb == part.b || nk > P.kb_m)
+            for (int e = tl; e < m * P.reck; e += T) {
+              const int j = e / P.reck;
+              ws[P.o_KE + e] = __ldg(a.recs_signed + ket0 + (int64_t)(part.k + (i0 + j) * part.nk) * P.reck +
+                                     (e - j * P.reck));
+            }
+          const RBatch bt{pb, 1, part.k, part.nk, nk};
+          compute_R_batch<CTA>(a, bra0, ket0, bt, i0, m, ws + P.o_KR, ws + P.o_KS, tl, mask);
+          for (int j = 0; j < m; ++j) {
+            const int dR = P.o_KR + j * P.rstride - P.o_R0, dE = P.o_KE + j * P.reck - P.o_reck;
+            run_step(P.kprog + grp.k1_off, grp.k1_n, ws, tl, T, false, dR, dE);
+            team_sync<CTA>(mask);
+            run_step(P.kprog + grp.k2_off, grp.k2_n, ws, tl, T, false, 0, dE);
+            team_sync<CTA>(mask);
+            run_step(P.kprog + grp.k3_off, grp.k3_n, ws, tl, T, i0 + j > 0, 0, dE);
+            team_sync<CTA>(mask);
+          }
+        }
+      } else for (int pk = part.k; pk < Kk; pk += part.nk) {
         if (P.cache_R != 1) {
           load_record(ws + P.o_reck, a.recs_signed + ket0 + (int64_t)pk * P.reck, P.reck, tl, T);
-          if (P.cache_R == 2) load_cached_R(P, ws, pb * Kk + pk, tl);
+          if (P.cache_R == 2) load_cached_R(P, ws, icache++, tl);
           team_sync<CTA>(mask);
           if (P.cache_R == 0) compute_R<CTA>(a, ws, tl, mask);
         }

@@ -164,6 +164,11 @@ struct PlanDev {
                                          // primitive quartets kept at o_Rc (rstride doubles each); 3 (solid-
                                          // harmonic plans): those of the current bra primitive; 0: R per group
   int32_t o_Rc, rstride;
+  // Batches of kb_m primitive quartets whose R tables are formed together (compute_R_batch): per batch slot a
+  // table at o_KR (rstride doubles) and a ket record at o_KE, working space at o_KS (kb_work doubles each).
+  // kb_m = 0: one primitive quartet at a time. Plans with cached tables (cache_R >= 2) batch the filling of
+  // their tables at o_Rc, with the working space alone.
+  int32_t kb_m, o_KR, o_KE, o_KS;
   int32_t reg;                           // launch the register kernel (store / digestion launches)
   int32_t has_out;                       // OUT region present (0: store-only plan, b23 writes global memory)
   // Solid-harmonic output (store = 2). The ket groups write their Cartesian columns [p|cd] to a
@@ -194,6 +199,10 @@ struct PlanDev {
   const uint16_t* colmap;
   const uint16_t* colinv;   // per group g: colinv[g * Nk + ket column] = its column in g, or 0xffff
 };
+
+// Working space of one primitive quartet in a batch of R tables: the odd levels of Eq. r, P - Q, T, prefactor and
+// -2 rho, and the Boys seeds.
+constexpr int kb_work(int L) { return tet(L) + 6 + L + 1; }
 
 // Host-side plan with its program arrays.
 struct Plan {

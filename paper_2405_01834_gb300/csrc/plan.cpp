@@ -230,6 +230,21 @@ bool validate_plan(const Plan& plan, std::string& err) {
       return false;
     }
   }
+  if (P.kb_m > 0) {
+    // the batch's tables and records lie after every other region; its working space there too, or in what is
+    // not in use while the tables are formed (never the records, OUT, or X between the batches of a bra primitive)
+    const long m = P.kb_m, work = m * kb_work(P.L);
+    const bool whole = P.cache_R >= 2 || m >= P.Kk;
+    const long end_other = P.o_OUT + (long)P.ncols_max * (P.has_out ? P.Nb : 0);
+    const long hi = P.cache_R >= 2 ? P.o_Rc : (whole ? P.o_OUT : P.o_X);
+    const bool inside = P.o_KS >= P.o_R0 + tet(P.L + 1) && P.o_KS + work <= hi;
+    if ((!inside && P.o_KS + work > W) ||
+        (P.cache_R < 2 && (P.o_KR < end_other || P.o_KE < P.o_KR + m * P.rstride || P.o_KE + m * P.reck > W ||
+                           (!inside && P.o_KS < P.o_KE + m * P.reck)))) {
+      err = "batch of R tables out of range";
+      return false;
+    }
+  }
   if (P.sph) {
     // the bra pass starts where the ket groups' region starts (R at level 0 stays below it), and the
     // [a][b'] pass of each column fits its C1 slot
@@ -592,6 +607,47 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
       }
     }
   }
+  // R tables in batches of primitive quartets (compute_R_batch)
+  if (key.Kb * key.Kk > 1) {
+    const int work = kb_work(P.L);
+    if (P.cache_R >= 2) {
+      // the tables are filled before anything else of the workspace is in use (cache_R == 3: of what a bra
+      // primitive's ket groups write); at least one at a time
+      const int n = (P.cache_R == 2 ? key.Kb : 1) * key.Kk;
+      P.o_KS = o_region;
+      P.kb_m = std::min(n, (P.o_Rc - o_region) / work);
+      if (P.kb_m < 1) {
+        P.kb_m = 1;
+        P.o_KS = (P.team_doubles + 1) & ~1;
+        P.team_doubles = (P.o_KS + work) | 1;
+      }
+    } else if (P.ngroups == 1 && !sph) {
+      const int base = (P.team_doubles + 1) & ~1;
+      // as many as the workspace may grow by: an SM's teams shall still hold 512 lanes (T: as chosen below, about
+      // 30 multiply-adds per lane and primitive quartet), or the workspace grow to 1.3 times
+      double per_prim = fma_k + 8.0 * (P.L + 1) + fma_b * P.Nk / key.Kk;
+      for (int n = 0; n < P.L; ++n) per_prim += tet(P.L - n + 1) - 1;
+      int t = 8;
+      while (t < 128 && 2 * t * 30.0 <= per_prim) t *= 2;
+      const int room = std::max((int)(0.3 * base), std::min(220 * 1024 / 512 * t, smem_budget_bytes) / 8 - base);
+      auto extra = [&](int m) {
+        const bool inside = m * work <= (m >= key.Kk ? P.o_OUT : P.o_X) - o_region;
+        return m * (P.rstride + P.reck) + (inside ? 0 : m * work);
+      };
+      int m = key.Kk;
+      while (m > 1 && extra(m) > room) --m;
+      // (teams of less than a warp synchronise cheaply, and their lanes are few enough for a single primitive's
+      // levels: [43|00] K = 36 on 16 lanes 0.73 ms without batches, 0.97 ms in batches of two. Batches over several
+      // bra primitives cost more teams per SM than they save: [00|61] K = 36 3.31 -> 3.82 ms)
+      if (m > 1 && t >= 32 && (base + extra(m)) * 8 <= smem_budget_bytes && base + extra(m) < 65536) {
+        P.kb_m = m;
+        P.o_KR = base;
+        P.o_KE = base + m * P.rstride;
+        P.o_KS = m * work <= (m >= key.Kk ? P.o_OUT : P.o_X) - o_region ? o_region : P.o_KE + m * P.reck;
+        P.team_doubles = (base + extra(m)) | 1;
+      }
+    }
+  }
   // inverse column maps: the digestion epilogue visits only the columns of its own K block
   plan.colinv.assign((size_t)P.ngroups * P.Nk, 0xffff);
   for (int gi = 0; gi < P.ngroups; ++gi)
@@ -706,7 +762,7 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
   // a team's chain: a barrier-separated step costs some 500 clocks of load and barrier latency, and each of
   // its lanes' multiply-adds about 24
   const double nrec_k = P.cache_R == 2 ? 0.0 : P.ngroups;   // R levels inside the group loop
-  P.cost_k = (float)(500.0 * (nrec_k * (P.L + 2) + 4.0 * P.ngroups) + 24.0 * (fma_k + nrec_k * fma_r) / P.T);
+  P.cost_k = (float)(500.0 * (nrec_k * (P.L + 2) / std::max(1, P.kb_m) + 4.0 * P.ngroups) + 24.0 * (fma_k + nrec_k * fma_r) / P.T);
   P.cost_b = (float)(500.0 * 2.0 * P.ngroups + 24.0 * fma_b * P.Nk / P.T);
   if (P.T * P.teams_per_cta > 1024 || (long)P.teams_per_cta * P.team_doubles * 8 > 227 * 1024) {
     err = "team shape exceeds the CTA limits";
