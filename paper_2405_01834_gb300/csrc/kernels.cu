@@ -81,7 +81,7 @@ __global__ void k_pair_records(BasisDev b0, BasisDev b1, const PrimPairJob* __re
   double* r = recs + jb.off;
   double* rs = recs_signed + jb.off;
   const double pref = ca * cb * exp(-za * zb * ab2 * ip);
-  const double hdr[kRecHeader] = {p, ip, P[0], P[1], P[2], pref, pref * ip, 0.0};
+  const double hdr[kRecHeader] = {p, ip, P[0], P[1], P[2], pref, pref * ip, zb * ip};
   for (int k = 0; k < kRecHeader; ++k) { r[k] = hdr[k]; rs[k] = hdr[k]; }
   // per-axis tables, E_00^0 = 1 (the exponential is in the prefactor)
   int tab = 0;  // etab size

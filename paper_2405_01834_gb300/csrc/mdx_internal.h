@@ -39,7 +39,7 @@ const std::vector<double>& rys_table();    // rys_table.cpp; built on first use
 // ----------------------------------------------------------------- records
 // Primitive-pair record: header of kRecHeader doubles, then the three per-axis
 // E tables (x, y, z). Header: [0] zeta_p, [1] 1/zeta_p, [2..4] P, [5] prefactor
-// c_a c_b exp(-zeta_a zeta_b |A-B|^2 / zeta_p), [6] the prefactor over zeta_p, [7] unused.
+// c_a c_b exp(-zeta_a zeta_b |A-B|^2 / zeta_p), [6] the prefactor over zeta_p, [7] zeta_b / zeta_p.
 constexpr int kRecHeader = 8;
 
 inline int etab_size(int la, int lb) {      // sum over a<=la, b<=lb of (a+b+1)

@@ -112,11 +112,163 @@ __device__ __forceinline__ double eprod(const double* ex, const double* ey, cons
   else return __ldg(ex) * __ldg(ey) * __ldg(ez);
 }
 
+// ---- contracted ket pairs [ps), [ds), [pp): sums of scaled R tables instead of one ket transform per primitive
+// With s = zeta_d / zeta_q, r = 1 / (2 zeta_q) and X = C - D of the pair, Q - C = -s X and Q - D = (1 - s) X, and every
+// Hermite coefficient E^cd_q of Eqs. E2rr1/E2rr2 is a polynomial in X with coefficients s^M (1-s)^N r^w, where q
+// of total order T takes w = T + (l_c + l_d - M - N - T) / 2. X is the same for all primitives of the pair, so
+//   [p|cd] = sum over (M, N, T), |q| = T of  c X^(M+N) S_MNT[p + q],   S_MNT[h] = sum_k (s^M (1-s)^N r^w)_k R_k[h],
+// and a primitive quartet costs the accumulation of the S tables (orders T .. L_b + T of R) in place of the whole ket
+// transform; the expansion runs once per bra primitive. FP64 instructions per primitive quartet: [fs|ps] 120 -> 54,
+// [dp|pp] 660 -> 160 (of about 360 and 870 with R and the Boys seeds). The E tables' cancellations are the same ones
+// (Q - C and Q - D enter as products of s with one distance, as accurate as the tables' own differences).
+template <int LC, int LD>
+struct KetSets {
+  static constexpr int n = 0, M[1] = {}, N[1] = {}, T[1] = {};
+};
+template <>
+struct KetSets<1, 0> {
+  static constexpr int n = 2, M[2] = {1, 0}, N[2] = {0, 0}, T[2] = {0, 1};
+};
+template <>
+struct KetSets<2, 0> {
+  static constexpr int n = 4, M[4] = {2, 0, 1, 0}, N[4] = {0, 0, 0, 0}, T[4] = {0, 0, 1, 2};
+};
+template <>
+struct KetSets<1, 1> {
+  static constexpr int n = 5, M[5] = {1, 0, 1, 0, 0}, N[5] = {1, 0, 0, 1, 0}, T[5] = {0, 0, 1, 1, 2};
+};
+// one term of [p|cd]: coef * monomial(X) * S_set[p + q]; monomials 1, X, Y, Z, XX, XY, XZ, YY, YZ, ZZ
+struct KetTerm {
+  int cd, set, q[3], mono, coef;
+};
+constexpr __host__ __device__ int binom(int n, int k) { return k == 0 || k == n ? 1 : binom(n - 1, k - 1) + binom(n - 1, k); }
+// ways in which k Gaussian coordinates become t Hermite indices and (k - t) / 2 contracted pairs
+constexpr __host__ __device__ int hermite_ways(int k, int t) {
+  int f = binom(k, t);
+  for (int i = k - t - 1; i > 1; i -= 2) f *= i;
+  return f;
+}
+constexpr __host__ __device__ int monomial(int x, int y, int z) {
+  if (x + y + z == 0) return 0;
+  if (x + y + z == 1) return x ? 1 : (y ? 2 : 3);
+  return x == 2 ? 4 : (x == 1 ? (y ? 5 : 6) : (y == 2 ? 7 : (y == 1 ? 8 : 9)));
+}
+constexpr int kKetTermsMax = 39;
+struct KetTermTable {
+  KetTerm t[kKetTermsMax];
+  int n;
+};
+template <int LC, int LD>
+constexpr __host__ __device__ KetTermTable ket_terms() {
+  KetTermTable r{};
+  using S = KetSets<LC, LD>;
+  for (int c = 0; c < ncart(LC); ++c)
+    for (int d = 0; d < ncart(LD); ++d)
+      for (int i = 0; i < S::n; ++i) {
+        const int C[3] = {cx(LC, c), cy(LC, c), cz(LC, c)}, D[3] = {cx(LD, d), cy(LD, d), cz(LD, d)};
+        // per axis: m of the c coordinates give Q - C, n of the d ones Q - D, t Hermite indices
+        for (int m0 = 0; m0 <= C[0]; ++m0) for (int m1 = 0; m1 <= C[1]; ++m1) for (int m2 = 0; m2 <= C[2]; ++m2)
+        for (int n0 = 0; n0 <= D[0]; ++n0) for (int n1 = 0; n1 <= D[1]; ++n1) for (int n2 = 0; n2 <= D[2]; ++n2)
+        for (int t0 = 0; t0 <= 2; ++t0) for (int t1 = 0; t1 <= 2; ++t1) for (int t2 = 0; t2 <= 2; ++t2) {
+          if (m0 + m1 + m2 != S::M[i] || n0 + n1 + n2 != S::N[i] || t0 + t1 + t2 != S::T[i]) continue;
+          const int k0 = C[0] - m0 + D[0] - n0, k1 = C[1] - m1 + D[1] - n1, k2 = C[2] - m2 + D[2] - n2;
+          if (k0 < t0 || k1 < t1 || k2 < t2 || ((k0 - t0) & 1) || ((k1 - t1) & 1) || ((k2 - t2) & 1)) continue;
+          int f = binom(C[0], m0) * binom(C[1], m1) * binom(C[2], m2) * binom(D[0], n0) * binom(D[1], n1) *
+                  binom(D[2], n2) * hermite_ways(k0, t0) * hermite_ways(k1, t1) * hermite_ways(k2, t2);
+          if ((S::M[i] + S::T[i]) & 1) f = -f;   // Q - C = -s X, and the ket sign (-1)^|q| of Eq. pq
+          r.t[r.n] = KetTerm{c * ncart(LD) + d, i, {t0, t1, t2}, monomial(m0 + n0, m1 + n1, m2 + n2), f};
+          ++r.n;
+        }
+      }
+  return r;
+}
+template <int LC, int LD>
+struct KetTerms {
+  static constexpr KetTermTable v = ket_terms<LC, LD>();
+};
+// S tables of a class: set i holds the orders T .. L_b + T at set_off(i); the sets of the first group go through
+// registers when the tables are expanded, the second group lies behind [p|cd] (see k_reg)
+template <int LA, int LB, int LC, int LD>
+struct KetPlan {
+  using S = KetSets<LC, LD>;
+  static constexpr int Lb = LA + LB, NX = nherm(Lb) * ncart(LC) * ncart(LD);
+  static constexpr bool XS = !reg_eligible(LA, LB, LC, LD);
+  static constexpr __host__ __device__ int set_size(int i) { return nherm(Lb + S::T[i]) - nherm(S::T[i] - 1); }
+  static constexpr __host__ __device__ int total() {
+    int s = 0;
+    for (int i = 0; i < S::n; ++i) s += set_size(i);
+    return s;
+  }
+  // beside R in registers, or in the shared-memory region of [p|cd] (in registers too they would leave half the
+  // warps: [fs|ps] K = 1,6,3,6 2.16 ms from shared memory, 2.56 from registers)
+  static constexpr bool in_regs = !XS;
+  // first group: the sets of the highest T first, as many as 96 doubles hold (all of them in registers)
+  static constexpr __host__ __device__ bool first(int i) {
+    if (in_regs) return true;
+    int used = 0;
+    bool in = false;
+    for (int k = S::n - 1; k >= 0; --k) {
+      const bool fits = used + set_size(k) <= 96;
+      if (fits) used += set_size(k);
+      if (k == i) in = fits;
+    }
+    return in;
+  }
+  static constexpr __host__ __device__ int first_size() {
+    int s = 0;
+    for (int i = 0; i < S::n; ++i) s += first(i) ? set_size(i) : 0;
+    return s;
+  }
+  static constexpr int second_at = NX > first_size() ? NX : first_size();
+  static constexpr __host__ __device__ int set_off(int i) {
+    int s = in_regs || first(i) ? 0 : second_at;
+    for (int k = 0; k < i; ++k) s += first(k) == first(i) ? set_size(k) : 0;
+    return s;
+  }
+  // doubles per thread of the shared [p|cd] region, without and with the S tables
+  static constexpr int plain = XS ? NX : 0;
+  static constexpr int region = XS ? (in_regs ? NX : second_at + total() - first_size()) : 0;
+};
+// position of (t, u, v), T <= t + u + v <= N, in the [t][u][v] simplex of order N without its orders below T <= 2
+constexpr __host__ __device__ int sidx(int N, int T, int t, int u, int v) {
+  return hidx(N, t, u, v) - (T == 0 ? 0 : (T == 1 ? 1 : 2 + (t + u >= 1) + (t >= 1)));
+}
+// 64-thread blocks of an SM by shared memory (doubles per thread)
+constexpr int xs_blocks(int doubles) { return 227 * 1024 / (doubles * kXsBlock * 8 + 1024); }
+// Classes that use the S tables: those that keep their blocks per SM, or nearly so ([ds|ds] 7 -> 6 blocks: 1.27 -> 1.18
+// ms); where the bigger region halves them ([dp|pp] store) the two forms take the same time. Not the [ds) kets of a
+// bra of total order 4 (205 doubles), whose expansion does not fit the registers
+template <int LA, int LB, int LC, int LD, bool DIGEST>
+constexpr bool ket_sums_eligible() {
+  if constexpr (KetSets<LC, LD>::n == 0) return false;
+  else {
+    using P = KetPlan<LA, LB, LC, LD>;
+    if (!P::XS) return true;
+    const int v = DIGEST ? ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD) : 0;
+    return P::total() <= 170 && 4 * xs_blocks(P::region + v) >= 3 * xs_blocks(P::plain + v);
+  }
+}
+// Blocks per SM that the registers are limited for: as many as the shared memory holds, up to what the kernel's
+// tables need (the expansion's first group, or R, and 60 registers beside them)
+template <int LA, int LB, int LC, int LD, bool DIGEST>
+constexpr int ket_sums_blocks() {
+  using P = KetPlan<LA, LB, LC, LD>;
+  if (!P::XS) return 2;
+  const int v = DIGEST ? ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD) : 0;
+  const int tab = P::first_size() > nherm(LA + LB + LC + LD) ? P::first_size() : nherm(LA + LB + LC + LD);
+  const int by_regs = 65536 / kXsBlock / (2 * tab + 60), by_smem = xs_blocks(P::region + v);
+  const int b = by_regs < by_smem ? by_regs : by_smem;
+  return b < 4 ? 4 : b;
+}
+// ket primitives per lane from which the expansion is paid back
+constexpr int kKetSumsMin = 3;
+
 // XS = false: R, [p|cd] and the shellset in registers (classes with
 // reg_eligible). XS = true: R in registers, [p|cd] and the shellset in shared
 // memory (classes with reg_xs_eligible, total angular momentum <= 6).
-template <int LA, int LB, int LC, int LD, bool DIGEST, bool XS>
-__global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch a) {
+// KS = true: contracted ket pairs by sums of scaled R tables (KetSets).
+template <int LA, int LB, int LC, int LD, bool DIGEST, bool XS, bool KS>
+__global__ void __launch_bounds__(XS ? kXsBlock : 128, KS ? ket_sums_blocks<LA, LB, LC, LD, DIGEST>() : 0) k_reg(const QuartetLaunch a) {
   constexpr int Lb = LA + LB, Lk = LC + LD, L = Lb + Lk;
   constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD);
   constexpr int Nb = NA * NB, Nk = NC * ND;
@@ -151,6 +303,35 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
     X.p = xs_smem + (VSH ? Nb * Nk : 0) * kXsBlock + threadIdx.x;
   }
   if constexpr (!XS) sfor<Nb * Nk>([&](auto i) { V[i] = 0.0; });
+  // KS: the S tables in registers or, before [p|cd] takes their place, in its shared-memory region; monomials of C - D
+  using KP = KetPlan<LA, LB, LC, LD>;
+  constexpr bool SSH = KS && !KP::in_regs;
+  constexpr int NS = KS ? KP::total() : 1;
+  TArr<SSH, NS> SR;
+  double mono[KS ? 10 : 1];
+  if constexpr (KS) {
+    if constexpr (SSH) SR.p = X.p;
+    const double* E10 = rk0 + kRecHeader + etab_off(LD, 1, 0);
+    if constexpr (LD > 0) {
+      const double* E01 = rk0 + kRecHeader + etab_off(LD, 0, 1);
+      sfor<3>([&](auto x) { mono[1 + x] = __ldg(E01 + x * EK) - __ldg(E10 + x * EK); });   // (Q - D) - (Q - C)
+    } else {
+      // from the primitive with the largest s: the error of X times any s is at most that of Q - C itself
+      int top = -1, at = 0;
+      for (int k = 0; k < Kk; ++k) {
+        const int h = __double2hiint(__ldg(rk0 + (int64_t)k * RK + 7));
+        if (h > top) { top = h; at = k; }
+      }
+      const double sm = __ldg(rk0 + (int64_t)at * RK + 7);
+      const double is = sm > 1e-290 ? -1.0 / sm : 0.0;
+      sfor<3>([&](auto x) { mono[1 + x] = __ldg(E10 + (int64_t)at * RK + x * EK) * is; });
+    }
+    mono[0] = 1.0;
+    if constexpr (Lk > 1) {
+      mono[4] = mono[1] * mono[1]; mono[5] = mono[1] * mono[2]; mono[6] = mono[1] * mono[3];
+      mono[7] = mono[2] * mono[2]; mono[8] = mono[2] * mono[3]; mono[9] = mono[3] * mono[3];
+    }
+  }
   double* const outq = DIGEST ? nullptr : a.out + (a.qout ? a.qout[q] : q * (int64_t)(Nb * Nk));
 
   for (int pb0 = 0; pb0 < Kb; pb0 += Sb) {
@@ -161,7 +342,13 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
     const double Px = __ldg(rb + 2), Py = __ldg(rb + 3), Pz = __ldg(rb + 4);
     // 2 pi^(5/2) * c_a c_b K_ab / zp (the ket part and 1/sqrt(zp+zq) per ket primitive)
     const double prefb = 34.986836655249725693 * __ldg(rb + 6);
-    sfor<HB * Nk>([&](auto i) { X[i] = 0.0; });
+    if constexpr (KS) {
+      sfor<KetSets<LC, LD>::n>([&](auto i) {
+        sfor<KP::set_size(i)>([&](auto h) { SR[KP::set_off(i) + h] = 0.0; });
+      });
+    } else {
+      sfor<HB * Nk>([&](auto i) { X[i] = 0.0; });
+    }
 
     for (int pk = live ? sk : Kk; pk < Kk; pk += Sk) {
       const double* __restrict__ rk = rk0 + (int64_t)pk * RK;
@@ -235,6 +422,31 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
         });
         R[0] = G[n];
       });
+      if constexpr (KS) {
+        using S = KetSets<LC, LD>;
+        const double zs = __ldg(rk + 7), zr = -__ldg(rk + kRecHeader + etab_off(LD, 1, 0) + 1);   // signed table: -r
+        sfor<S::n>([&](auto i) {
+          constexpr int M1 = S::M[i], N1 = S::N[i], T1 = S::T[i];
+          constexpr int w = T1 + (Lk - M1 - N1 - T1) / 2, N = Lb + T1;
+          double f = 1.0;
+          if constexpr (N1 > 0) f = 1.0 - zs;
+          else if constexpr (M1 > 0) f = zs;
+          if constexpr (M1 + N1 > 1) f *= zs;
+          if constexpr (M1 + N1 > 0 && w > 0) f *= zr;
+          else if constexpr (w > 0) f = zr;
+          if constexpr (w > 1) f *= zr;
+          sfor<N + 1>([&](auto t) {
+            sfor<N + 1 - t>([&](auto u) {
+              sfor<N + 1 - t - u>([&](auto v) {
+                if constexpr (t + u + v >= T1) {
+                  constexpr int o = KP::set_off(i) + sidx(N, T1, t, u, v);
+                  SR[o] = fma(f, R[hidx(L, t, u, v)], SR[o]);
+                }
+              });
+            });
+          });
+        });
+      } else
       // ket transform: X[p][cd] += sum_{tau,nu,phi} Ex Ey Ez (signed tables) R[p + q]
       sfor<NC>([&](auto c) {
         sfor<ND>([&](auto d) {
@@ -268,6 +480,40 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128) k_reg(const QuartetLaunch
           });
         });
       });
+    }
+    if constexpr (KS) {
+      // [p|cd] from the S tables: those of the first group pass through registers, since [p|cd] takes their place
+      using KT = KetTerms<LC, LD>;
+      constexpr int NF = KP::first_size(), second = NS - NF;
+      double F[SSH ? NF : 1];
+      if constexpr (SSH) sfor<NF>([&](auto i) { F[i] = SR[i]; });
+      auto expand = [&](auto grp2) {   // the terms of one group; the second adds to the first
+        sfor<Lb + 1>([&](auto t) {
+          sfor<Lb + 1 - t>([&](auto u) {
+            sfor<Lb + 1 - t - u>([&](auto v) {
+              constexpr int h = hidx(Lb, t, u, v) * Nk;
+              double x[Nk];
+              sfor<Nk>([&](auto cd) { x[cd] = grp2 ? X[h + cd] : 0.0; });
+              sfor<KT::v.n>([&](auto k) {
+                constexpr KetTerm e = KT::v.t[k];
+                if constexpr (KP::first(e.set) != (grp2 == 1)) {
+                  constexpr int T = KetSets<LC, LD>::T[e.set];
+                  constexpr int o = KP::set_off(e.set) + sidx(Lb + T, T, t + e.q[0], u + e.q[1], v + e.q[2]);
+                  double y;
+                  if constexpr (SSH && !(grp2 == 1)) y = F[o];
+                  else y = SR[o];
+                  if constexpr (e.mono == 0 && e.coef == 1) x[e.cd] += y;
+                  else if constexpr (e.mono == 0 && e.coef == -1) x[e.cd] -= y;
+                  else x[e.cd] = fma((double)e.coef * mono[e.mono], y, x[e.cd]);
+                }
+              });
+              sfor<Nk>([&](auto cd) { X[h + cd] = x[cd]; });
+            });
+          });
+        });
+      };
+      expand(Ic<0>{});
+      if constexpr (second > 0) expand(Ic<1>{});
     }
     // bra transform: V[ab][cd] += sum_{t,u,v} Ex Ey Ez X[tuv][cd]
     if constexpr (XS) {
@@ -476,21 +722,21 @@ inline void split_of(int64_t nq, int concurrent, int Kb, int Kk, double ck, doub
     }
 }
 
-template <int LA, int LB, int LC, int LD>
-cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
+// The instance of one epilogue: with the S tables of the ket pair where the class has them and each lane runs
+// enough ket primitives.
+template <int LA, int LB, int LC, int LD, bool DIGEST>
+cudaError_t launch_reg_epilogue(const QuartetLaunch& a, unsigned grid, cudaStream_t s) {
   constexpr bool XS = !reg_eligible(LA, LB, LC, LD);
   constexpr int bs = XS ? kXsBlock : 128;
-  constexpr int Nk = ncart(LC) * ncart(LD);
-  // shared memory per block: [p|cd] (and, with the digestion epilogue, the shellset) of every thread
-  constexpr size_t shm_x = XS ? (size_t)nherm(LA + LB) * Nk * kXsBlock * sizeof(double) : 0;
-  constexpr size_t shm_d = XS ? (size_t)ncart(LA) * ncart(LB) * Nk * kXsBlock * sizeof(double) + shm_x : 0;
-  QuartetLaunch a = a0;
-  constexpr double ck = reg_body_size(LA, LB, LC, LD, false) + 8.0 * (LA + LB + LC + LD + 1) + 80.0;
-  constexpr double cb = reg_body_size(LA, LB, LC, LD) - reg_body_size(LA, LB, LC, LD, false);
-  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
-  const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
-  if (grid > 0x7fffffff) return cudaErrorInvalidValue;
-  if constexpr (shm_d > 48 * 1024) {
+  // shared memory per block: [p|cd] or the S tables (and, with the digestion epilogue, the shellset) of every thread
+  using P = KetPlan<LA, LB, LC, LD>;
+  constexpr int v = XS && DIGEST ? ncart(LA) * ncart(LB) * ncart(LC) * ncart(LD) : 0;
+  constexpr size_t shm = (size_t)(P::plain + v) * kXsBlock * sizeof(double);
+  constexpr bool KS = ket_sums_eligible<LA, LB, LC, LD, DIGEST>();
+  constexpr size_t shm_s = KS ? (size_t)(P::region + v) * kXsBlock * sizeof(double) : shm;
+  auto* const plain = k_reg<LA, LB, LC, LD, DIGEST, XS, false>;
+  auto* const sums = k_reg<LA, LB, LC, LD, DIGEST, XS, KS>;
+  if constexpr (shm_s > 48 * 1024) {
     // opt in to more than 48 KB of dynamic shared memory, once per instance and device
     static bool attr[kRegMaxDevices] = {};
     int dev = 0;
@@ -498,18 +744,31 @@ cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kRegMaxDevices) return cudaErrorInvalidDevice;
     if (!attr[dev]) {
-      e = cudaFuncSetAttribute(k_reg<LA, LB, LC, LD, true, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)shm_d);
-      if (e == cudaSuccess && shm_x > 48 * 1024)
-        e = cudaFuncSetAttribute(k_reg<LA, LB, LC, LD, false, XS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)shm_x);
+      e = cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_s);
       if (e != cudaSuccess) return e;
       attr[dev] = true;
     }
   }
-  if (a.D) k_reg<LA, LB, LC, LD, true, XS><<<(unsigned)grid, bs, shm_d, s>>>(a);
-  else k_reg<LA, LB, LC, LD, false, XS><<<(unsigned)grid, bs, shm_x, s>>>(a);
+  const int per = (a.plan.Kk + (1 << a.split_k) - 1) >> a.split_k;   // ket primitives per lane
+  if (KS && per >= kKetSumsMin) sums<<<grid, bs, shm_s, s>>>(a);
+  else plain<<<grid, bs, shm, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int LA, int LB, int LC, int LD>
+cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
+  constexpr bool XS = !reg_eligible(LA, LB, LC, LD);
+  constexpr int bs = XS ? kXsBlock : 128;
+  constexpr int Nk = ncart(LC) * ncart(LD);
+  QuartetLaunch a = a0;
+  constexpr double ck = reg_body_size(LA, LB, LC, LD, false) + 8.0 * (LA + LB + LC + LD + 1) + 80.0;
+  constexpr double cb = reg_body_size(LA, LB, LC, LD) - reg_body_size(LA, LB, LC, LD, false);
+  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
+  const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
+  if (grid > 0x7fffffff) return cudaErrorInvalidValue;
+  return a.D ? launch_reg_epilogue<LA, LB, LC, LD, true>(a, (unsigned)grid, s)
+             : launch_reg_epilogue<LA, LB, LC, LD, false>(a, (unsigned)grid, s);
 }
 
 using RegLaunchFn = cudaError_t (*)(const QuartetLaunch&, cudaStream_t);
