@@ -1439,8 +1439,13 @@ struct XPrep {
 };
 
 // fill = false: counts only (X.d_quart stays unset).
+// by_l: the shell of the higher angular momentum comes first in its pair. Digestion and gradient treat the two shells
+// of a pair alike, so (ps| and (sp| pairs become one class: half the pair classes, fewer and larger launches, and kets
+// [ps), [ds) that the register kernel contracts as sums (exchange of 5 atoms 79.0 -> 75.7 ms, gradient of 3 atoms
+// 118.9 -> 100.4 ms, 8-molecule batched exchange 52.7 -> 51.5 ms). Otherwise the higher shell index comes first
+// (mdx_exchange_screen, whose work model counts the classes of that order).
 mdx_status exchange_screen(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs, const double* Q, int64_t n_pairs,
-                           double tau, const double* D, XPrep& X, cudaStream_t s, bool fill = true) {
+                           double tau, const double* D, XPrep& X, cudaStream_t s, bool by_l, bool fill = true) {
   if (!basis || !basis->ao_off) return fail(c, MDX_EINVAL, "basis needs ao_off");
   mdx_status st = fetch_basis(c, basis, X.hb, s);
   if (st != MDX_OK) return st;
@@ -1470,6 +1475,7 @@ mdx_status exchange_screen(mdx_ctx* c, const mdx_basis* basis, const int32_t* pa
     if (!(hq[p] >= 0.0)) return fail(c, MDX_EINVAL, "Schwarz factors must be >= 0");
     if (i < j) std::swap(i, j);
     if (!seen.emplace((int64_t)i * hb.n + j, 1).second) return fail(c, MDX_EINVAL, "shell pair listed twice");
+    if (by_l && hb.l[i] < hb.l[j]) std::swap(i, j);
     X.pl[p] = XPrep::P4{i, j, hq[p], hb.l[i], hb.l[j], hb.nprim[i] * hb.nprim[j], p};
   }
   std::stable_sort(X.pl.begin(), X.pl.end(), [](const XPrep::P4& a, const XPrep::P4& b) {
@@ -1593,7 +1599,7 @@ mdx_status mdx_exchange(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs
   if (n_pairs < 0 || !D || !K || (n_pairs > 0 && (!pairs || !Q)) || !(tau >= 0.0))
     return fail(c, MDX_EINVAL, "invalid arguments");
   XPrep X;
-  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s);
+  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true);
   if (st != MDX_OK) return st;
   cudaError_t e = cudaMemsetAsync(K, 0, (size_t)X.nao * X.nao * sizeof(double), s);
   if (e == cudaSuccess && energy) e = cudaMemsetAsync(energy, 0, sizeof(double), s);
@@ -1673,7 +1679,7 @@ mdx_status mdx_exchange_screen(mdx_ctx* c, const mdx_basis* basis, const int32_t
   if (model_flops) *model_flops = 0.0;
   XPrep X;
   // count first; list only when the caller asked for it and it fits
-  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, false);
+  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, false, false);
   if (st != MDX_OK) return st;
   *n_kept = X.nq;
   if (model_flops) {
@@ -1711,7 +1717,7 @@ mdx_status mdx_exchange_grad(mdx_ctx* c, const mdx_basis* basis, const int32_t* 
     return fail(c, MDX_EINVAL, "invalid arguments");
   if (!basis || !basis->atom) return fail(c, MDX_EINVAL, "basis needs atom");
   XPrep X;
-  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s);
+  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true);
   if (st != MDX_OK) return st;
   const HostBasis& hb = X.hb;
   const int32_t n = hb.n;
@@ -2023,12 +2029,16 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
   const mdx_basis sb{ntot, (int32_t)EX.size(), X->l, X->nprim, X->prim_off, X->ao_off, nullptr, X->center, X->exps,
                      X->coefs};
   X->sb = sb;
-  // all shell pairs i >= j of every molecule, sorted by (molecule, class)
+  // all shell pairs of every molecule, the shell of the higher angular momentum first (see exchange_screen), sorted
+  // by (molecule, class)
   struct PP { int32_t i, j, m, li, lj, K; };
   std::vector<PP> pl;
   for (int m = 0; m < n_mol; ++m)
     for (int32_t i = shell_first[m]; i < shell_first[m + 1]; ++i)
-      for (int32_t j = shell_first[m]; j <= i; ++j) pl.push_back(PP{i, j, m, L[i], L[j], NP[i] * NP[j]});
+      for (int32_t j = shell_first[m]; j <= i; ++j) {
+        const bool swap = L[i] < L[j];
+        pl.push_back(PP{swap ? j : i, swap ? i : j, m, std::max(L[i], L[j]), std::min(L[i], L[j]), NP[i] * NP[j]});
+      }
   std::stable_sort(pl.begin(), pl.end(), [](const PP& a, const PP& b) {
     if (a.m != b.m) return a.m < b.m;
     if (a.li != b.li) return a.li < b.li;
