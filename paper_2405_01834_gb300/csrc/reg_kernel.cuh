@@ -263,6 +263,79 @@ constexpr int ket_sums_blocks() {
 // ket primitives per lane from which the expansion is paid back
 constexpr int kKetSumsMin = 3;
 
+// Boys seeds of one primitive quartet and its Hermite integrals [tuv] of orders 0 .. L (Eqs. 0m, r) in R.
+template <int L>
+__device__ __forceinline__ void hermite_R(const double* __restrict__ boys, double zp, double zq, double PQx, double PQy,
+                                          double PQz, double pref, double* R) {
+  const double s = zp + zq;
+  const double R2 = PQx * PQx + PQy * PQy + PQz * PQz;
+  // Boys seeds G[m] = (-2 rho)^m pref F_m(T), m = 0..L (Eq. 0m), rho = zp zq / s, T = rho R^2, without a
+  // branch between the table and the asymptotic form F_m(T) = Gamma(m+1/2) / (2 T^(m+1/2)):
+  // with y = 1/sqrt(s) below T = 64 and y = 1/sqrt(zp zq R^2) above, and b = -2 zp zq y^2,
+  //   G[m] = C y b^m f_m,  f_m = F_m(T) below and Gamma(m+1/2)/2 above,
+  // and the table's last row holds the constants (T is 1 there, a grid point). The branch had cost a
+  // quarter of the FP64 issue slots of [ps|ss] (warps whose quartets lie on both sides run both).
+  // exp(-T) / (2 T F_m) is below 1e-20 from T = 64 on for m <= 6. With this, the one-term E tables and the
+  // coefficient 1 of Eq. r (40,000 quartets): [ss|ss] K = 6,6,6,6 5.74 -> 4.09 ms, [ps|ss] K = 3,6,6,6
+  // 4.22 -> 2.88 ms, [dp|ps] K = 1,3,3,6 1.55 -> 1.39 ms.
+  const double zz2 = -2.0 * zp * zq;              // -2 zp zq
+  const double c2 = zz2 * R2;                  // -2 zp zq R^2
+  const int hc = __double2hiint(c2) & 0x7fffffff;
+  const bool far = hc >= __double2hiint(s) + (7 << 20);   // 2 zp zq R^2 >= 128 s, by the exponents
+  // zp zq R^2 = c2 / -2: sign off, exponent less one
+  const double y = rsqrt(far ? __hiloint2double(hc - (1 << 20), __double2loint(c2)) : s);
+  const double y2 = y * y;
+  const double T2 = c2 * y2;                   // -2 T
+  // nearest grid point of spacing 1/16: the low word of T + 1.5 2^48
+  const double tm = fma(T2, -0.5, 422212465065984.0);
+  const double nd = fma(T2, 0.5, tm - 422212465065984.0);   // T0 - T
+  const int i = far ? kBoysNgrid - 1 : min(__double2loint(tm) & 0x7fffffff, kBoysNgrid - 1);
+  const double2* row = reinterpret_cast<const double2*>(boys + (size_t)i * kBoysRow);
+  double G[L + 1];
+  {
+    const double bm = zz2 * y2;
+    double pw = pref * y;
+    sfor<L + 1>([&](auto m) {
+      const double2 c01 = __ldg(row + 4 * m), c23 = __ldg(row + 4 * m + 1);
+      const double2 c45 = __ldg(row + 4 * m + 2), c67 = __ldg(row + 4 * m + 3);
+      double f = fma(c67.y, nd, c67.x);
+      f = fma(f, nd, c45.y);
+      f = fma(f, nd, c45.x);
+      f = fma(f, nd, c23.y);
+      f = fma(f, nd, c23.x);
+      f = fma(f, nd, c01.y);
+      f = fma(f, nd, c01.x);
+      G[m] = pw * f;
+      if constexpr (m < L) pw *= bm;
+    });
+  }
+  // R^(n)_tuv for n = L..0 in one array indexed in the order-L simplex:
+  // level n overwrites orders N = L-n..1 from the top down (an entry reads
+  // orders N-1 and N-2 of level n+1, not yet overwritten), then [000]
+  R[0] = G[L];
+  sfor<L>([&](auto k) {
+    constexpr int n = L - 1 - k;
+    sfor<L - n>([&](auto j) {
+      constexpr int N = L - n - j;
+      sfor<N + 1>([&](auto t) {
+        sfor<N + 1 - t>([&](auto u) {
+          constexpr int v = N - t - u;
+          double val;
+          if constexpr (v > 0) {
+            val = raise<v>(PQz, R[hidx(L, t, u, v - 1)], [&] { return R[hidx(L, t, u, v - 2)]; });
+          } else if constexpr (u > 0) {
+            val = raise<u>(PQy, R[hidx(L, t, u - 1, 0)], [&] { return R[hidx(L, t, u - 2, 0)]; });
+          } else {
+            val = raise<t>(PQx, R[hidx(L, t - 1, 0, 0)], [&] { return R[hidx(L, t - 2, 0, 0)]; });
+          }
+          R[hidx(L, t, u, v)] = val;
+        });
+      });
+    });
+    R[0] = G[n];
+  });
+}
+
 // XS = false: R, [p|cd] and the shellset in registers (classes with
 // reg_eligible). XS = true: R in registers, [p|cd] and the shellset in shared
 // memory (classes with reg_xs_eligible, total angular momentum <= 6).
@@ -338,7 +411,7 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128, KS ? ket_sums_blocks<LA, 
     const bool live = pb0 + sb < Kb;   // a lane past the last bra primitive adds zeros to the group's sums
     const int pb = live ? pb0 + sb : 0;
     const double* __restrict__ rb = rb0 + (int64_t)pb * RB;
-    const double zp = __ldg(rb), zpm2 = -2.0 * zp;
+    const double zp = __ldg(rb);
     const double Px = __ldg(rb + 2), Py = __ldg(rb + 3), Pz = __ldg(rb + 4);
     // 2 pi^(5/2) * c_a c_b K_ab / zp (the ket part and 1/sqrt(zp+zq) per ket primitive)
     const double prefb = 34.986836655249725693 * __ldg(rb + 6);
@@ -354,74 +427,8 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128, KS ? ket_sums_blocks<LA, 
       const double* __restrict__ rk = rk0 + (int64_t)pk * RK;
       const double zq = __ldg(rk);
       const double PQx = Px - __ldg(rk + 2), PQy = Py - __ldg(rk + 3), PQz = Pz - __ldg(rk + 4);
-      const double s = zp + zq;
-      const double R2 = PQx * PQx + PQy * PQy + PQz * PQz;
-      // Boys seeds G[m] = (-2 rho)^m pref F_m(T), m = 0..L (Eq. 0m), rho = zp zq / s, T = rho R^2, without a
-      // branch between the table and the asymptotic form F_m(T) = Gamma(m+1/2) / (2 T^(m+1/2)):
-      // with y = 1/sqrt(s) below T = 64 and y = 1/sqrt(zp zq R^2) above, and b = -2 zp zq y^2,
-      //   G[m] = C y b^m f_m,  f_m = F_m(T) below and Gamma(m+1/2)/2 above,
-      // and the table's last row holds the constants (T is 1 there, a grid point). The branch had cost a
-      // quarter of the FP64 issue slots of [ps|ss] (warps whose quartets lie on both sides run both).
-      // exp(-T) / (2 T F_m) is below 1e-20 from T = 64 on for m <= 6. With this, the one-term E tables and the
-      // coefficient 1 of Eq. r (40,000 quartets): [ss|ss] K = 6,6,6,6 5.74 -> 4.09 ms, [ps|ss] K = 3,6,6,6
-      // 4.22 -> 2.88 ms, [dp|ps] K = 1,3,3,6 1.55 -> 1.39 ms.
-      const double zz2 = zpm2 * zq;                // -2 zp zq
-      const double c2 = zz2 * R2;                  // -2 zp zq R^2
-      const int hc = __double2hiint(c2) & 0x7fffffff;
-      const bool far = hc >= __double2hiint(s) + (7 << 20);   // 2 zp zq R^2 >= 128 s, by the exponents
-      // zp zq R^2 = c2 / -2: sign off, exponent less one
-      const double y = rsqrt(far ? __hiloint2double(hc - (1 << 20), __double2loint(c2)) : s);
-      const double y2 = y * y;
-      const double T2 = c2 * y2;                   // -2 T
-      // nearest grid point of spacing 1/16: the low word of T + 1.5 2^48
-      const double tm = fma(T2, -0.5, 422212465065984.0);
-      const double nd = fma(T2, 0.5, tm - 422212465065984.0);   // T0 - T
-      const int i = far ? kBoysNgrid - 1 : min(__double2loint(tm) & 0x7fffffff, kBoysNgrid - 1);
-      const double2* row = reinterpret_cast<const double2*>(boys + (size_t)i * kBoysRow);
-      double G[L + 1];
-      {
-        const double bm = zz2 * y2;
-        double pw = prefb * __ldg(rk + 6) * y;
-        sfor<L + 1>([&](auto m) {
-          const double2 c01 = __ldg(row + 4 * m), c23 = __ldg(row + 4 * m + 1);
-          const double2 c45 = __ldg(row + 4 * m + 2), c67 = __ldg(row + 4 * m + 3);
-          double f = fma(c67.y, nd, c67.x);
-          f = fma(f, nd, c45.y);
-          f = fma(f, nd, c45.x);
-          f = fma(f, nd, c23.y);
-          f = fma(f, nd, c23.x);
-          f = fma(f, nd, c01.y);
-          f = fma(f, nd, c01.x);
-          G[m] = pw * f;
-          if constexpr (m < L) pw *= bm;
-        });
-      }
-      // R^(n)_tuv for n = L..0 in one array indexed in the order-L simplex:
-      // level n overwrites orders N = L-n..1 from the top down (an entry reads
-      // orders N-1 and N-2 of level n+1, not yet overwritten), then [000]
       double R[HL];
-      R[0] = G[L];
-      sfor<L>([&](auto k) {
-        constexpr int n = L - 1 - k;
-        sfor<L - n>([&](auto j) {
-          constexpr int N = L - n - j;
-          sfor<N + 1>([&](auto t) {
-            sfor<N + 1 - t>([&](auto u) {
-              constexpr int v = N - t - u;
-              double val;
-              if constexpr (v > 0) {
-                val = raise<v>(PQz, R[hidx(L, t, u, v - 1)], [&] { return R[hidx(L, t, u, v - 2)]; });
-              } else if constexpr (u > 0) {
-                val = raise<u>(PQy, R[hidx(L, t, u - 1, 0)], [&] { return R[hidx(L, t, u - 2, 0)]; });
-              } else {
-                val = raise<t>(PQx, R[hidx(L, t - 1, 0, 0)], [&] { return R[hidx(L, t - 2, 0, 0)]; });
-              }
-              R[hidx(L, t, u, v)] = val;
-            });
-          });
-        });
-        R[0] = G[n];
-      });
+      hermite_R<L>(boys, zp, zq, PQx, PQy, PQz, prefb * __ldg(rk + 6), R);
       if constexpr (KS) {
         using S = KetSets<LC, LD>;
         const double zs = __ldg(rk + 7), zr = -__ldg(rk + kRecHeader + etab_off(LD, 1, 0) + 1);   // signed table: -r
@@ -722,6 +729,105 @@ inline void split_of(int64_t nq, int concurrent, int Kb, int Kk, double ck, doub
     }
 }
 
+// Uncontracted shellsets of the classes below: one warp per block, one thread per quartet, everything in registers. The
+// columns [p|cd] are formed one at a time and go through the bra transform at once, so that neither [p|cd] nor the
+// shellset is ever whole; the products of the bra's E tables are formed once. The shared-memory variant holds [p|cd]
+// of a class ([pp|pp]: 46 KB per 64 threads, 8 warps per SM), which made 1.3 waves of the sweep's 50,176 quartets and
+// kept the FP64 pipe 51 % busy; here 12 warps fit and the launch is one wave. 50,176 quartets: [pp|pp] 151 -> 103 us,
+// [ds|pp] 122 -> 91, [sp|sg] 130 -> 116; 100 quartets: 62 -> 48, 54 -> 44, 58 -> 54 us (pair records included).
+template <int LA, int LB>
+struct BraTerms {   // Hermite terms of the Cartesian bra pairs, pair by pair
+  static constexpr __host__ __device__ int size(int ia, int ib) {
+    return (cx(LA, ia) + cx(LB, ib) + 1) * (cy(LA, ia) + cy(LB, ib) + 1) * (cz(LA, ia) + cz(LB, ib) + 1);
+  }
+  static constexpr __host__ __device__ int off(int ia, int ib) {
+    int s = 0;
+    for (int k = 0; k < ia * ncart(LB) + ib; ++k) s += size(k / ncart(LB), k % ncart(LB));
+    return s;
+  }
+  static constexpr __host__ __device__ int total() { return off(ncart(LA), 0); }
+};
+// R and the bra products within 72 doubles, and a body that compiles quickly
+template <int LA, int LB, int LC, int LD>
+constexpr bool single_eligible() {
+  return !reg_eligible(LA, LB, LC, LD) && nherm(LA + LB + LC + LD) + BraTerms<LA, LB>::total() <= 72 &&
+         reg_body_size(LA, LB, LC, LD) <= 1000;
+}
+template <int LA, int LB, int LC, int LD>
+__global__ void __launch_bounds__(32, 12) k_reg_single(const QuartetLaunch a) {
+  constexpr int Lb = LA + LB, L = Lb + LC + LD;
+  constexpr int NA = ncart(LA), NB = ncart(LB), NC = ncart(LC), ND = ncart(LD), Nk = NC * ND;
+  constexpr int EB = etab_size(LA, LB), EK = etab_size(LC, LD);
+  using BT = BraTerms<LA, LB>;
+  const int64_t q = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  if (q >= a.nq) return;
+  const int2 qp = a.qpairs[q];
+  const double* __restrict__ rb = a.recs + a.pair_rec[qp.x + a.bra_var_off];
+  const double* __restrict__ rk = a.recs_signed + a.pair_rec[qp.y + a.ket_var_off];
+  double* const outq = a.out + (a.qout ? a.qout[q] : q * (int64_t)(NA * NB * Nk));
+  double R[nherm(L)];
+  hermite_R<L>(a.boys, __ldg(rb), __ldg(rk), __ldg(rb + 2) - __ldg(rk + 2), __ldg(rb + 3) - __ldg(rk + 3),
+               __ldg(rb + 4) - __ldg(rk + 4), 34.986836655249725693 * __ldg(rb + 6) * __ldg(rk + 6), R);
+  double B[BT::total()];
+  sfor<NA>([&](auto ia) {
+    sfor<NB>([&](auto ib) {
+      constexpr int ax = cx(LA, ia), ay = cy(LA, ia), az = cz(LA, ia);
+      constexpr int bx = cx(LB, ib), by = cy(LB, ib), bz = cz(LB, ib);
+      constexpr int nx = ax + bx + 1, ny = ay + by + 1, nz = az + bz + 1, o = BT::off(ia, ib);
+      const double* Ex = rb + kRecHeader + etab_off(LB, ax, bx);
+      const double* Ey = rb + kRecHeader + EB + etab_off(LB, ay, by);
+      const double* Ez = rb + kRecHeader + 2 * EB + etab_off(LB, az, bz);
+      sfor<nx * ny * nz>([&](auto k) {
+        B[o + k] = eprod<nx, ny, nz>(Ex + k / (ny * nz), Ey + k / nz % ny, Ez + k % nz);
+      });
+    });
+  });
+  sfor<NC>([&](auto c) {
+    sfor<ND>([&](auto d) {
+      double X[nherm(Lb)];
+      {
+        constexpr int ex = cx(LC, c), ey = cy(LC, c), ez = cz(LC, c);
+        constexpr int fx = cx(LD, d), fy = cy(LD, d), fz = cz(LD, d);
+        constexpr int nx = ex + fx + 1, ny = ey + fy + 1, nz = ez + fz + 1;
+        const double* Ex = rk + kRecHeader + etab_off(LD, ex, fx);
+        const double* Ey = rk + kRecHeader + EK + etab_off(LD, ey, fy);
+        const double* Ez = rk + kRecHeader + 2 * EK + etab_off(LD, ez, fz);
+        double E[nx * ny * nz];
+        sfor<nx * ny * nz>([&](auto k) {
+          E[k] = eprod<nx, ny, nz>(Ex + k / (ny * nz), Ey + k / nz % ny, Ez + k % nz);
+        });
+        sfor<Lb + 1>([&](auto t) {
+          sfor<Lb + 1 - t>([&](auto u) {
+            sfor<Lb + 1 - t - u>([&](auto v) {
+              double acc = 0.0;
+              sfor<nx * ny * nz>([&](auto k) {
+                const double r = R[hidx(L, t + k / (ny * nz), u + k / nz % ny, v + k % nz)];
+                if constexpr (nx * ny * nz == 1) acc = r;
+                else if constexpr (k == 0) acc = E[k] * r;
+                else acc = fma(E[k], r, acc);
+              });
+              X[hidx(Lb, t, u, v)] = acc;
+            });
+          });
+        });
+      }
+      sfor<NA>([&](auto ia) {
+        sfor<NB>([&](auto ib) {
+          constexpr int ny = cy(LA, ia) + cy(LB, ib) + 1, nz = cz(LA, ia) + cz(LB, ib) + 1, n = BT::size(ia, ib), o = BT::off(ia, ib);
+          double acc = 0.0;
+          sfor<n>([&](auto k) {
+            const double x = X[hidx(Lb, k / (ny * nz), k / nz % ny, k % nz)];
+            if constexpr (n == 1) acc = x;
+            else if constexpr (k == 0) acc = B[o] * x;
+            else acc = fma(B[o + k], x, acc);
+          });
+          outq[(ia * NB + ib) * Nk + c * ND + d] = acc;
+        });
+      });
+    });
+  });
+}
+
 // The instance of one epilogue: with the S tables of the ket pair where the class has them and each lane runs
 // enough ket primitives.
 template <int LA, int LB, int LC, int LD, bool DIGEST>
@@ -748,6 +854,12 @@ cudaError_t launch_reg_epilogue(const QuartetLaunch& a, unsigned grid, cudaStrea
       if (e == cudaSuccess) e = cudaFuncSetAttribute(sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_s);
       if (e != cudaSuccess) return e;
       attr[dev] = true;
+    }
+  }
+  if constexpr (!DIGEST && single_eligible<LA, LB, LC, LD>()) {
+    if (a.plan.Kb * a.plan.Kk == 1) {
+      k_reg_single<LA, LB, LC, LD><<<(unsigned)((a.nq + 31) / 32), 32, 0, s>>>(a);
+      return cudaGetLastError();
     }
   }
   const int per = (a.plan.Kk + (1 << a.split_k) - 1) >> a.split_k;   // ket primitives per lane
