@@ -40,11 +40,11 @@ UNIT = "GFLOP/s (Table-1 model FLOPs)"
 # peak that is reported beside the measured one
 FP64_FLOP_PER_CLK_SM = 4.0
 CHUNK_BYTES = 2 << 30
-# DRAM bytes (read + write) per [ii|ii] quartet of one k_quartets launch of the benchmark (456 quartets,
-# autotuned plan): ncu --nvtx --nvtx-include "mdx_batch_run/" -k regex:k_quartets -c 1 --metrics
+# DRAM bytes (read + write) per [ii|ii] quartet of one k_rys launch of the benchmark (456 quartets):
+# ncu --nvtx --nvtx-include "mdx_batch_run/" -k regex:k_rys -c 1 --metrics
 # dram__bytes_read.sum,dram__bytes_write.sum on `bench.py --classes 6 --n-bra 24 --n-ket 19 --steps 1
-# --warmup 3 --no-cpu --no-e2e`: 5,659,966,464 B read + 7,211,322,368 B written
-NCU_DRAM_BYTES_PER_II_QUARTET = (5659966464 + 7211322368) / 456
+# --warmup 3 --no-cpu --no-e2e`: 1,000,510,464 B read + 2,647,006,464 B written
+NCU_DRAM_BYTES_PER_II_QUARTET = (1000510464 + 2647006464) / 456
 
 
 def parse():
@@ -982,7 +982,7 @@ def main():
     traffic = None
     if NCU_DRAM_BYTES_PER_II_QUARTET is not None and l == 6:
         traffic = round(NCU_DRAM_BYTES_PER_II_QUARTET * len(q) / len(batches))
-    roofline = {"bound": "alu", "kernel": "k_quartets %s" % CLASS_NAMES[l], "achieved": round(achieved, 4),
+    roofline = {"bound": "alu", "kernel": "%s %s" % ("k_rys" if l > 1 else "k_reg_single", CLASS_NAMES[l]), "achieved": round(achieved, 4),
                 "peak": round(peak_gflops * 1e-3, 4), "unit": "TFLOP/s", "frac": round(achieved / (peak_gflops * 1e-3), 4),
                 "traffic": traffic, "traffic_unit": "DRAM bytes read + written per launch (ncu)",
                 "algorithmic_flops_per_launch": per_launch_exec,

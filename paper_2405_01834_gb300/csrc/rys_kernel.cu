@@ -14,7 +14,8 @@
 // shared-memory loads per pair of them free; lanes run over the ket components, so that stores are whole
 // lines and a row of a table is read without bank conflicts. The tables of one quartet stay in shared memory up to
 // [gg|gg] (135 KB); larger classes keep them in a global area per block (749 KB at [ii|ii], L2) and copy the rows
-// of one bra component a at a time (107 KB at [ii|ii], two blocks per SM).
+// of one bra component a at a time (107 KB of the block's 163 KB at [ii|ii]: one block of 16 warps per SM, FP64 pipe 85 %
+// busy).
 // Contracted quartets keep the step programs, which fold the ket primitives before the bra steps.
 #include <algorithm>
 #include <utility>
