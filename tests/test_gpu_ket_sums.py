@@ -24,6 +24,9 @@ def test_contracted_kets(lq, K):
         s = 2 * n + 2 * k + (k // 6) % 2
         o = b.prim_off[s]
         b.exps[o: o + b.nprim[s]] *= 1e-10
+    for k in range(2, n, 6):            # negative exponents on the second shell, within those of the first
+        i, j = (b.exps[b.prim_off[s]: b.prim_off[s] + b.nprim[s]] for s in (2 * n + 2 * k, 2 * n + 2 * k + 1))
+        j[:] = -0.01 * i.min()
     eng, db = mdx.Engine(0), mdx.DeviceBasis(b)
     assert eng.plan_info(*lq, K[0] * K[1], K[2] * K[3]).register_kernel == 1
     v, off = eng.eri4(db, q)
