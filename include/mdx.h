@@ -215,7 +215,11 @@ mdx_status mdx_batch_offsets(mdx_ctx* ctx, const mdx_batch* batch, int64_t* out_
  * 0m, r, pq, ket-from-hermite, bra-from-hermite). Writes the integrals at the
  * batch's offsets in `out` (out_capacity doubles). No host synchronisation
  * and no allocation; n_launches (may be NULL) receives the number of kernels
- * enqueued. Kernel-side errors surface at the next mdx_sync. */
+ * enqueued. Kernel-side errors surface at the next mdx_sync.
+ * Runs of one Cartesian batch into different outputs may overlap on the GPU
+ * (runs on several streams, captured graphs replayed side by side), also
+ * with runs of other batches. Runs of one solid-harmonic batch must not: they
+ * share the batch's staging area. */
 mdx_status mdx_batch_run(mdx_ctx* ctx, mdx_batch* batch, double* out, int64_t out_capacity, int32_t* n_launches,
                          void* stream);
 

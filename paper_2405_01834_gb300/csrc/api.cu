@@ -36,11 +36,26 @@ struct NvtxRange {
   ~NvtxRange() { nvtxRangePop(); }
 };
 
+// Axis tables of the Rys classes that keep them in global memory: `areas` of `stride` doubles, as many as their blocks
+// that the GPU holds at a time, each taken by a block while it runs (`used`). The prepared batches of a context
+// share one (114 MB for [ii|ii]); it goes with the last batch that uses it.
+struct RysAreas {
+  double* tab = nullptr;
+  int32_t* used = nullptr;
+  int64_t stride = 0;
+  int areas = 0;
+  ~RysAreas() {
+    cudaFree(tab);
+    cudaFree(used);
+  }
+};
+
 struct mdx_ctx {
   int device = 0;
   std::string last_error;
   double* d_boys = nullptr;
   double* d_rys = nullptr;                // Rys nodes and weights, uploaded when a class first needs them
+  std::weak_ptr<RysAreas> rys_areas;      // the batches' newest areas
   uint32_t* d_rprog = nullptr;
   int32_t* d_rprog_off = nullptr;
   int* d_err = nullptr;
@@ -166,6 +181,29 @@ mdx_status need_rys_table(mdx_ctx* c) {
   return MDX_OK;
 }
 
+// Areas of at least `stride` doubles, at least `n` of them: the batches' present ones, or new ones that serve both.
+mdx_status need_rys_areas(mdx_ctx* c, int64_t stride, int n, std::shared_ptr<RysAreas>* out, cudaStream_t s) {
+  const std::shared_ptr<RysAreas> cur = c->rys_areas.lock();
+  if (cur && cur->stride >= stride && cur->areas >= n) {
+    *out = cur;
+    return MDX_OK;
+  }
+  auto a = std::make_shared<RysAreas>();
+  a->stride = cur ? std::max(stride, cur->stride) : stride;
+  a->areas = cur ? std::max(n, cur->areas) : n;
+  if (cudaMalloc(&a->tab, (size_t)a->areas * a->stride * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&a->used, (size_t)a->areas * sizeof(int32_t)) != cudaSuccess) {
+    cudaGetLastError();
+    return fail(c, MDX_ENOMEM, "Rys table area allocation failed");
+  }
+  cudaError_t e = cudaMemsetAsync(a->used, 0, (size_t)a->areas * sizeof(int32_t), s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // runs on other streams come after it
+  if (e != cudaSuccess) return cuda_fail(c, e, "Rys table area");
+  c->rys_areas = a;
+  *out = a;
+  return MDX_OK;
+}
+
 mdx_status check_device_error(mdx_ctx* c, cudaStream_t s) {
   int h = 0;
   cudaError_t e = cudaMemcpyAsync(&h, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -255,6 +293,10 @@ struct mdx_batch {
   double* cart = nullptr;
   double* xg = nullptr;
   int64_t nxg = 0;                // doubles allocated at xg
+  // Rys classes with tables in global memory: the areas of prepared batches, or (one-shot calls, which never overlap)
+  // context workspace at rys_tab, one area per block
+  std::shared_ptr<RysAreas> rys;
+  double* rys_tab = nullptr;
   struct Range { Plan* plan; int64_t begin, count; ClassKey key; Plan* splan; int grid; };
   std::vector<Range> ranges;
   std::vector<std::pair<double, int32_t>> order;   // (model FLOPs, range), heaviest first: launch order
@@ -316,6 +358,16 @@ void batch_free(mdx_batch* b) {
     cudaFree(b->cqoff); cudaFree(b->cart); cudaFree(b->xg);
   }
   delete b;
+}
+
+// The Rys fields of a launch of range r.
+void set_rys(const mdx_ctx* c, const mdx_batch* B, const mdx_batch::Range& r, QuartetLaunch& a) {
+  a.rys = c->d_rys;
+  if (!r.plan->d.ry_stash) return;
+  a.rys_tab = B->rys ? B->rys->tab : B->rys_tab;
+  a.rys_used = B->rys ? B->rys->used : nullptr;
+  a.rys_stride = B->rys ? B->rys->stride : r.plan->d.ry_table;
+  a.rys_areas = B->rys ? B->rys->areas : r.grid;
 }
 
 template <typename T>
@@ -454,6 +506,8 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
   qp_sorted.reserve(bt.qp.size());
   qoff_sorted.reserve(bt.qp.size());
   int64_t cart_total = 0, xg_total = 0;
+  int64_t rys_total = 0, rys_stride = 0;   // tables in global memory: of one launch, of one block
+  int rys_resident = 0;
   mdx_status st;
   for (auto& kv : classes) {
     const int64_t b = (int64_t)qp_sorted.size();
@@ -470,9 +524,12 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
     double fma = plan->exec_fma;
     if (!sph && plan->d.rys) {
       if ((st = need_rys_table(c)) != MDX_OK) return st;
-      cudaError_t e = rys_grid(plan->d, cnt, &grid);
+      int resident = 0;
+      cudaError_t e = rys_grid(plan->d, cnt, &grid, &resident);
       if (e != cudaSuccess) return cuda_fail(c, e, "Rys launch shape");
-      xg_total = std::max<int64_t>(xg_total, (int64_t)grid * plan->d.ry_table);
+      rys_total = std::max<int64_t>(rys_total, (int64_t)grid * plan->d.ry_table);
+      rys_stride = std::max<int64_t>(rys_stride, plan->d.ry_table);
+      rys_resident = std::max(rys_resident, resident);
       fma = plan->rys_fma;
     }
     ClassKey ks = kv.first;
@@ -531,14 +588,10 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
       return fail(c, MDX_ENOMEM, "record allocation failed");
     }
   }
-  if (!sph && xg_total > 0) {   // the global axis tables of the largest Rys classes
-    if (call_ws) {
-      if ((st = ensure(c, "call_rys", (size_t)xg_total, &B->xg, s)) != MDX_OK) return st;
-    } else if (cudaMalloc(&B->xg, xg_total * sizeof(double)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(c, MDX_ENOMEM, "Rys table area allocation failed");
-    }
-    B->nxg = xg_total;
+  if (rys_total > 0) {   // the global axis tables of the largest Rys classes
+    if (call_ws) st = ensure(c, "call_rys", (size_t)rys_total, &B->rys_tab, s);
+    else st = need_rys_areas(c, rys_stride, rys_resident, &B->rys, s);
+    if (st != MDX_OK) return st;
   }
   if (sph) {
     if ((st = dev_upload(c, cqoff, &B->cqoff, s)) != MDX_OK) return st;
@@ -596,9 +649,8 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
       ++nl;
       continue;
     }
-    if (!B->sph && r.plan->d.ry_stash) {   // one area of axis tables for all of them: one stream
-      a.rys = c->d_rys;
-      a.sph_scratch = B->xg;
+    if (!B->sph && r.plan->d.ry_stash) {   // tables in global memory: one after the other
+      set_rys(c, B, r, a);
       fan.load[0] += B->order[i].first;
       e = launch_rys(a, r.grid, s);
       ++nl;
@@ -606,7 +658,7 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
     }
     const cudaStream_t rs = fan.stream(fan.pick(B->order[i].first));
     if (!B->sph && r.plan->d.rys) {
-      a.rys = c->d_rys;
+      set_rys(c, B, r, a);
       e = launch_rys(a, r.grid, rs);
       ++nl;
       continue;
@@ -1287,8 +1339,7 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
       a.pair_rec = b->pair_rec;
       a.recs = b->recs;
       a.recs_signed = b->recs_s;
-      a.rys = c->d_rys;
-      a.sph_scratch = b->xg;
+      set_rys(c, b, r, a);
       a.out = out;
       a.err = c->d_err;
       for (int rep = 0; rep < 2; ++rep) {

@@ -76,6 +76,12 @@ struct QuartetLaunch {
   int32_t part_b, part_k;
   // solid-harmonic launches (plan.sph): global staging, xg_doubles per team of the launch grid
   double* sph_scratch;
+  // Rys kernel (plan.ry_stash): areas of rys_stride doubles for the axis tables. With rys_used (one word per area,
+  // zero when free) a block takes a free one of the rys_areas while it runs; without, block b uses area b.
+  double* rys_tab;
+  int32_t* rys_used;
+  int64_t rys_stride;
+  int32_t rys_areas;
 };
 
 static_assert(sizeof(QuartetLaunch) % sizeof(int) == 0, "descriptor copied word by word");
@@ -104,9 +110,9 @@ cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s);
 // grid * teams_per_cta * xg_doubles doubles.
 cudaError_t sph_grid(const PlanDev& P, int64_t nq, int* grid);
 cudaError_t launch_quartets_sph(const QuartetLaunch& a, int grid, cudaStream_t s);
-// Rys kernel (plan.rys, store epilogue): rys_grid gives the grid for nq quartets; with plan.ry_stash, a.sph_scratch
-// must hold grid * ry_table doubles.
-cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid);
+// Rys kernel (plan.rys, store epilogue): rys_grid gives the grid for nq quartets and, with plan.ry_stash, the number
+// of its blocks that the GPU holds at a time (0 otherwise); the areas at a.rys_tab hold ry_table doubles or more each.
+cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid, int* resident);
 cudaError_t launch_rys(const QuartetLaunch& a, int grid, cudaStream_t s);
 cudaError_t rys_attributes_init();
 // Writes zeros over n output ranges given as (offset, doubles) pairs (screened-out shellsets).

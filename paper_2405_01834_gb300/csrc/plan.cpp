@@ -278,6 +278,7 @@ static void plan_rys(Plan& plan) {
   // [61|00] 627 -> 432 us, [22|22] 2.08 -> 1.42 ms, [ff|ff] 4.02 -> 2.40 ms, [ii|ii] 27.5 -> 14.8 ms, 3-center
   // [6|10] 476 -> 378 us, [3|33] 6.48 -> 1.62 ms, [6|66] 11.6 -> 4.63 ms; no class of L >= 7 was slower.
   if (n > kRysMax || plan.rys_fma > 0.97 * plan.exec_fma) return;
+  // records, nodes and weights, one-dimensional functions, index words (and one for the block's table area)
   const int fixed = P.recb + P.reck + 2 * n + 3 * (P.L + 1) * n + ((P.Nb + P.Nk + nab1 + ncd1 + 1) / 2 + 1);
   auto doubles = [&](int cw, int rows) {
     return fixed + 3 * (P.Lb + 1) * n * cw * (P.ld + 1) + 3 * rows * n * ncd1;

@@ -13,7 +13,7 @@
 // kernel is bound by the FP64 pipe (an SM starts a warp's FP64 instruction every 19 clocks), which leaves three
 // shared-memory loads per pair of them free; lanes run over the ket components, so that stores are whole
 // lines and a row of a table is read without bank conflicts. The tables of one quartet stay in shared memory up to
-// [gg|gg] (135 KB); larger classes keep them in a global area per block (749 KB at [ii|ii], L2) and copy the rows
+// [gg|gg] (135 KB); larger classes keep them in a global area per resident block (749 KB at [ii|ii], L2) and copy the rows
 // of one bra component a at a time (107 KB of the block's 163 KB at [ii|ii]: one block of 16 warps per SM, FP64 pipe 85 %
 // busy).
 // Contracted quartets keep the step programs, which fold the ket primitives before the bra steps.
@@ -33,6 +33,22 @@ __device__ __forceinline__ int2 component(int l, int k) {
   int i = 0;
   while (k > i) k -= ++i;   // x = l - i, and y runs from i down
   return make_int2(l - i, i - k);
+}
+
+// A free area of the axis tables for this block. Launches that share the areas may overlap on the GPU (runs of a
+// batch on several streams, other batches, replayed graphs): there are as many areas as blocks that can be
+// resident together, so one is always free, and the search starts at the block's own (the first try succeeds unless
+// launches overlap). -1 after a bounded search.
+__device__ int take_area(int32_t* used, int n, int first) {
+  for (int round = 0; round < 4096; ++round)
+    for (int i = 0; i < n; ++i) {
+      const int k = first + i < n ? first + i : first + i - n;
+      if (atomicCAS(used + k, 0, 1) == 0) {
+        __threadfence();   // the last holder's accesses come before this block's
+        return k;
+      }
+    }
+  return -1;
 }
 
 template <int NR>
@@ -60,8 +76,12 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
   uint32_t* cdt = abt + Nb;                                     // columns of cd
   uint32_t* rowE = cdt + Nk;                                    // per one-axis ab: E block start, length
   uint32_t* colE = rowE + nab1;                                 // per one-axis cd
+  int* area = reinterpret_cast<int*>(colE + ncd1);              // of the tables in global memory
   const bool stash = P.ry_stash != 0;
-  double* gtab = stash ? a.sph_scratch + (int64_t)blockIdx.x * P.ry_table : tab;
+  if (stash && tid == 0) {
+    *area = a.rys_used ? take_area(a.rys_used, a.rys_areas, (int)(blockIdx.x % (unsigned)a.rys_areas)) : (int)blockIdx.x;
+    if (*area < 0) atomicExch(a.err, kDevTimeout);
+  }
 
   for (int e = tid; e < Nb; e += T) {
     const int ia = e / nb, ib = e - ia * nb;
@@ -85,6 +105,9 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
     const int x = e / (ld + 1), y = e - x * (ld + 1);
     colE[e] = (uint32_t)eoff(ld, x, y) | (uint32_t)(x + y + 1) << 16;
   }
+  __syncthreads();
+  if (stash && *area < 0) return;
+  double* gtab = stash ? a.rys_tab + *area * a.rys_stride : tab;
   const int EB = (P.recb - kRecHeader) / 3, EK = (P.reck - kRecHeader) / 3;   // one axis of a record's tables
   // (the record is padded to an even length: the table length is the integer part)
 
@@ -204,6 +227,13 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
       }
     }
   }
+  if (stash && a.rys_used) {
+    __syncthreads();   // every thread has read its tables
+    if (tid == 0) {
+      __threadfence();
+      atomicExch(a.rys_used + *area, 0);
+    }
+  }
 }
 
 using RysKernel = void (*)(const QuartetLaunch);
@@ -227,7 +257,8 @@ cudaError_t rys_attributes_init() {
   return cudaSuccess;
 }
 
-cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid) {
+cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid, int* resident) {
+  *resident = 0;
   if (!P.ry_stash) {
     *grid = (int)std::min<int64_t>(nq, 0x7fffffff);
     return cudaSuccess;
@@ -238,7 +269,8 @@ cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid) {
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nq, (int64_t)std::max(1, bps) * sms));
+  *resident = std::max(1, bps) * sms;
+  *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nq, *resident));
   return cudaSuccess;
 }
 
@@ -246,7 +278,9 @@ cudaError_t launch_rys(const QuartetLaunch& a, int grid, cudaStream_t s) {
   if (a.nq <= 0) return cudaSuccess;
   const PlanDev& P = a.plan;
   const RysKernel k = rys_kernel(P.rys);
-  if (!k || !a.rys || a.D || a.grad || grid < 1 || (P.ry_stash && !a.sph_scratch)) return cudaErrorInvalidValue;
+  if (!k || !a.rys || a.D || a.grad || grid < 1) return cudaErrorInvalidValue;
+  if (P.ry_stash && (!a.rys_tab || a.rys_stride < P.ry_table || a.rys_areas < (a.rys_used ? 1 : grid)))
+    return cudaErrorInvalidValue;
   k<<<grid, P.ry_threads, (size_t)P.ry_doubles * sizeof(double), s>>>(a);
   return cudaGetLastError();
 }
