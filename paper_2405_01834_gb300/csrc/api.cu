@@ -164,7 +164,9 @@ mdx_status get_plan(mdx_ctx* c, const ClassKey& k, Plan** out, cudaStream_t s) {
   return MDX_OK;
 }
 
-mdx_status need_rys_table(mdx_ctx* c) {
+// (cudaMemcpy from pageable memory returns once the data is staged and runs on the legacy default stream, which
+// non-blocking streams do not wait for: copied on `s`, and waited for, so that every later launch comes after it)
+mdx_status need_rys_table(mdx_ctx* c, cudaStream_t s) {
   if (c->d_rys) return MDX_OK;
   const std::vector<double>& tab = rys_table();
   double* p = nullptr;
@@ -172,7 +174,8 @@ mdx_status need_rys_table(mdx_ctx* c) {
     cudaGetLastError();
     return fail(c, MDX_ENOMEM, "Rys table allocation failed");
   }
-  const cudaError_t e = cudaMemcpy(p, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpyAsync(p, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     cudaFree(p);
     return cuda_fail(c, e, "Rys table upload");
@@ -523,7 +526,7 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
     int grid = 0;
     double fma = plan->exec_fma;
     if (!sph && plan->d.rys) {
-      if ((st = need_rys_table(c)) != MDX_OK) return st;
+      if ((st = need_rys_table(c, s)) != MDX_OK) return st;
       int resident = 0;
       cudaError_t e = rys_grid(plan->d, cnt, &grid, &resident);
       if (e != cudaSuccess) return cuda_fail(c, e, "Rys launch shape");
@@ -837,6 +840,8 @@ mdx_status mdx_create(mdx_ctx** ctx, int device) {
     return MDX_ECUDA;
   if (cudaMalloc(&c->d_err, sizeof(int)) != cudaSuccess) return MDX_ENOMEM;
   if (cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess) return MDX_ECUDA;
+  // the copies above are ordered on the legacy default stream only (see need_rys_table)
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return MDX_ECUDA;
   bool streams = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < mdx_ctx::kAux && streams; ++i)
     streams = cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking) == cudaSuccess &&

@@ -75,7 +75,8 @@ mdx_status setup(int dev, DevState& st) {
   o += align256(doff.size() * sizeof(int32_t));
   if (cudaMemcpy(st.boys, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(st.rprog, dec.data(), dec.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(st.rprog_off, doff.data(), doff.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaMemcpy(st.rprog_off, doff.data(), doff.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // non-blocking streams do not wait for the copies
     cudaGetLastError();
     return MDX_ECUDA;
   }
