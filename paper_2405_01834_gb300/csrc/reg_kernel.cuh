@@ -389,14 +389,16 @@ __global__ void __launch_bounds__(XS ? kXsBlock : 128, KS ? ket_sums_blocks<LA, 
       const double* E01 = rk0 + kRecHeader + etab_off(LD, 0, 1);
       sfor<3>([&](auto x) { mono[1 + x] = __ldg(E01 + x * EK) - __ldg(E10 + x * EK); });   // (Q - D) - (Q - C)
     } else {
-      // from the primitive with the largest |s|: the error of X times any s is at most that of Q - C itself
+      // from the primitive with the largest |s|: the error of X times any s is at most that of Q - C itself.
+      // (Q - C below 1e-140 X is nothing beside 1 / zeta_q's terms; dividing its rounding by such an s would give an X
+      // whose square is infinite)
       int top = -1, at = 0;
       for (int k = 0; k < Kk; ++k) {
         const int h = __double2hiint(__ldg(rk0 + (int64_t)k * RK + 7)) & 0x7fffffff;
         if (h > top) { top = h; at = k; }
       }
       const double sm = __ldg(rk0 + (int64_t)at * RK + 7);
-      const double is = fabs(sm) > 1e-290 ? -1.0 / sm : 0.0;
+      const double is = fabs(sm) > 1e-140 ? -1.0 / sm : 0.0;
       sfor<3>([&](auto x) { mono[1 + x] = __ldg(E10 + (int64_t)at * RK + x * EK) * is; });
     }
     mono[0] = 1.0;
