@@ -395,11 +395,14 @@ mdx_status dev_upload(mdx_ctx* c, const std::vector<T>& v, T** out, cudaStream_t
 // makes the caller's stream wait for all of them. While a stream capture that
 // the caller's stream does not belong to holds an auxiliary stream (a caller
 // that captures on one stream and launches on another), everything stays on
-// the caller's stream.
+// the caller's stream. `width`, the streams that the launches can use, decides how much of the GPU each takes
+// (QuartetLaunch::concurrent): it depends on their number alone, so that the order of the sums, and the results' bits, do
+// not depend on what else is being captured.
 struct Fanout {
   mdx_ctx* c;
   cudaStream_t s;
   int n = 0;   // auxiliary streams in use
+  int width = 1;
   double load[mdx_ctx::kAux + 1] = {};
   cudaStream_t stream(int i) const { return i == 0 ? s : c->aux[i - 1]; }
   static cudaError_t capture_id(cudaStream_t st, unsigned long long* id) {
@@ -411,6 +414,7 @@ struct Fanout {
   }
   cudaError_t fork(size_t launches) {
     const int want = (int)std::min<size_t>(mdx_ctx::kAux, launches > 0 ? launches - 1 : 0);
+    width = want + 1;
     if (want == 0) return cudaSuccess;
     unsigned long long own = 0, other = 0;
     cudaError_t e = capture_id(s, &own);
@@ -643,7 +647,7 @@ mdx_status batch_run(mdx_ctx* c, mdx_batch* B, double* out, int32_t* nlaunch, cu
     a.rprog_off = c->d_rprog_off;
     a.out = out;
     a.err = c->d_err;
-    a.concurrent = fan.n + 1;
+    a.concurrent = fan.width;
     if (B->sph && r.splan) {   // solid harmonics folded into the transforms
       a.plan = r.splan->d;
       a.sph_scratch = B->xg;
@@ -1705,7 +1709,7 @@ mdx_status mdx_exchange(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs
                      });
     Fanout fan{c, s};
     e = fan.fork(jobs_k.size());
-    for (size_t i = 0; i < jobs_k.size(); ++i) jobs_k[i].second.concurrent = fan.n + 1;
+    for (size_t i = 0; i < jobs_k.size(); ++i) jobs_k[i].second.concurrent = fan.width;
     for (size_t i = 0; i < jobs_k.size() && e == cudaSuccess; ++i)
       e = launch_quartets(jobs_k[i].second, fan.stream(fan.pick(jobs_k[i].first)));
     const cudaError_t ej = fan.join();
@@ -1929,7 +1933,7 @@ mdx_status mdx_exchange_grad(mdx_ctx* c, const mdx_basis* basis, const int32_t* 
   e = fan.fork(gjobs.size());
   for (size_t j = 0; j < gjobs.size() && e == cudaSuccess; ++j) {
     GradJob& g = gjobs[j];
-    g.a.concurrent = fan.n + 1;
+    g.a.concurrent = fan.width;
     const int si = fan.pick(g.work);
     const cudaStream_t gs = fan.stream(si);
     if (g.chunk == 0) {
@@ -2414,7 +2418,7 @@ mdx_status mdx_xbatch_run(mdx_ctx* c, mdx_xbatch* xb, int32_t persistent, int32_
       }
       for (size_t i = 0; i < xb->order.size() && e == cudaSuccess; ++i) {
         QuartetLaunch a = xb->launches[xb->order[i].second];
-        a.concurrent = fan.n + 1;
+        a.concurrent = fan.width;
         if (persistent == 2 && !xb->is_reg[xb->order[i].second]) continue;
         e = launch_quartets(a, fan.stream(fan.pick(xb->order[i].first)));
         ++nl;

@@ -69,7 +69,7 @@ struct QuartetLaunch {
   const double* const* mol_D;
   double* const* mol_K;
   const int32_t* mol_nao;
-  int32_t concurrent;        // launches that run beside this one (streams in use; 0: alone)
+  int32_t concurrent;        // launches that can run side by side with it, itself included (0: alone)
   // register kernel: 2^(split_b + split_k) lanes share a quartet's primitives (set by its launcher)
   int32_t split_b, split_k;
   // team kernel: part_b x part_k teams share a quartet's primitive pairs (set by launch_quartets)
