@@ -1503,9 +1503,9 @@ struct XPrep {
 // of a pair alike, so (ps| and (sp| pairs become one class: half the pair classes, fewer and larger launches, and kets
 // [ps), [ds) that the register kernel contracts as sums (exchange of 5 atoms 79.0 -> 75.7 ms, gradient of 3 atoms
 // 118.9 -> 100.4 ms, 8-molecule batched exchange 52.7 -> 51.5 ms). Otherwise the higher shell index comes first
-// (mdx_exchange_screen, whose work model counts the classes of that order).
+// (mdx_exchange_screen, whose list and work model are grouped by the classes of that order).
 mdx_status exchange_screen(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs, const double* Q, int64_t n_pairs,
-                           double tau, const double* D, XPrep& X, cudaStream_t s, bool by_l, bool fill = true) {
+                           double tau, const double* D, XPrep& X, cudaStream_t s, bool by_l, bool fill) {
   if (!basis || !basis->ao_off) return fail(c, MDX_EINVAL, "basis needs ao_off");
   mdx_status st = fetch_basis(c, basis, X.hb, s);
   if (st != MDX_OK) return st;
@@ -1659,7 +1659,7 @@ mdx_status mdx_exchange(mdx_ctx* c, const mdx_basis* basis, const int32_t* pairs
   if (n_pairs < 0 || !D || !K || (n_pairs > 0 && (!pairs || !Q)) || !(tau >= 0.0))
     return fail(c, MDX_EINVAL, "invalid arguments");
   XPrep X;
-  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true);
+  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true, true);
   if (st != MDX_OK) return st;
   cudaError_t e = cudaMemsetAsync(K, 0, (size_t)X.nao * X.nao * sizeof(double), s);
   if (e == cudaSuccess && energy) e = cudaMemsetAsync(energy, 0, sizeof(double), s);
@@ -1757,7 +1757,7 @@ mdx_status mdx_exchange_screen(mdx_ctx* c, const mdx_basis* basis, const int32_t
   if (!kept || X.nq == 0) return check_device_error(c, s);
   if (X.nq > kept_capacity) return fail(c, MDX_ECAPACITY, "kept-quartet capacity too small");
   XPrep X2;
-  if ((st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X2, s, true)) != MDX_OK) return st;
+  if ((st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X2, s, false, true)) != MDX_OK) return st;
   if (X2.nq != X.nq) return fail(c, MDX_EDEVICE, "screening counts differ between passes");
   cudaError_t e = launch_map_pairs(X2.d_quart, X2.nq, X2.d_orig, kept, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1777,7 +1777,7 @@ mdx_status mdx_exchange_grad(mdx_ctx* c, const mdx_basis* basis, const int32_t* 
     return fail(c, MDX_EINVAL, "invalid arguments");
   if (!basis || !basis->atom) return fail(c, MDX_EINVAL, "basis needs atom");
   XPrep X;
-  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true);
+  mdx_status st = exchange_screen(c, basis, pairs, Q, n_pairs, tau, D, X, s, true, true);
   if (st != MDX_OK) return st;
   const HostBasis& hb = X.hb;
   const int32_t n = hb.n;
