@@ -350,7 +350,8 @@ mdx_status mdx_xbatch_create(mdx_ctx* ctx, int32_t n_mol, const mdx_basis* bases
                              double* const* K, double tau, mdx_xbatch** xbatch, void* stream);
 
 /* Kept quartets, persistent work items, per-class launches and the Table-1
- * model FLOPs of the kept shellsets of a batch (any pointer may be NULL). */
+ * model FLOPs of the kept shellsets of a batch, counted as
+ * mdx_exchange_screen counts them (any pointer may be NULL). */
 mdx_status mdx_xbatch_info(const mdx_xbatch* xbatch, int64_t* n_quartets, int64_t* n_items,
                            int32_t* n_class_launches, double* model_flops);
 
@@ -377,8 +378,10 @@ mdx_status mdx_xbatch_autotune(mdx_ctx* ctx, mdx_xbatch* xbatch, int64_t max_tri
 
 /* Per-class launch i of a batch (0 <= i < n_class_launches): its class
  * lk = {la, lb, lc, ld, K_ab, K_cd} (K = primitive pairs of the bra / ket
- * shell pairs), its kept quartets and their Table-1 model FLOPs (any output
- * pointer may be NULL). MDX_EINVAL for an index out of range. */
+ * shell pairs; the shell of the higher angular momentum first in each pair),
+ * its kept quartets and their Table-1 model FLOPs as mdx_exchange_screen
+ * counts them (any output pointer may be NULL). MDX_EINVAL for an index out
+ * of range. */
 mdx_status mdx_xbatch_launch_info(const mdx_xbatch* xbatch, int32_t i, int32_t* lk, int64_t* n_quartets,
                                   double* model_flops);
 

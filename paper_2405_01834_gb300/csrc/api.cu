@@ -333,7 +333,7 @@ struct mdx_xbatch {
   std::vector<ClassKey> lkey;          // class of each per-class launch
   std::vector<double> lflops;          // its Table-1 model FLOPs
   std::vector<char> is_reg;            // per-class launches that run a register kernel
-  std::vector<std::pair<double, int32_t>> order;   // (model FLOPs, launch), heaviest first: launch order
+  std::vector<std::pair<double, int32_t>> order;   // (model FLOPs of the class as launched, launch), heaviest first
   QuartetLaunch* d_plaunches = nullptr;
   WorkItem* items = nullptr;
   WorkItem* items_team = nullptr;
@@ -2126,6 +2126,8 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
   if ((st = dev_upload(c, pmol, &X->pmol, s)) != MDX_OK) return st;
   int32_t* d_pclass;
   if ((st = upload(c, "xb_pclass", pclass_raw, &d_pclass, s)) != MDX_OK) return st;
+  std::vector<int32_t> class_flag(np);   // 2 class + 1 where the shells are not in index order
+  for (int64_t p = 0; p < np; ++p) class_flag[p] = 2 * pclass_raw[p] + (pl[p].i < pl[p].j ? 1 : 0);
   if (np > 0x7fffffff) return fail(c, MDX_EUNSUPPORTED, "too many shell pairs");
   // Schwarz factors and primitive-pair records of every pair (records stay with the batch)
   std::vector<int64_t> prec(np);
@@ -2266,6 +2268,32 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
       if (e == cudaSuccess) e = launch_screen(sa, true, s);
       if (e != cudaSuccess) return cuda_fail(c, e, "screening");
     }
+    // The work model counts a quartet as mdx_exchange_screen does, by the classes of the shells in index order, the
+    // higher one as bra: the model is not symmetric in bra and ket, and the launches' classes may have them the
+    // other way round
+    std::vector<unsigned long long> ocounts((size_t)nbucket * 4, 0);
+    if (X->nq > 0) {
+      unsigned long long* d_oc;
+      int32_t* d_cf;
+      if ((st = upload(c, "xb_class_flag", class_flag, &d_cf, s)) != MDX_OK) return st;
+      if ((st = ensure(c, "xb_ocounts", ocounts.size(), &d_oc, s)) != MDX_OK) return st;
+      e = cudaMemsetAsync(d_oc, 0, ocounts.size() * sizeof(unsigned long long), s);
+      if (e == cudaSuccess) e = launch_order_counts(X->quart, X->nq, d_cf, d_oc, s);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(ocounts.data(), d_oc, ocounts.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) return cuda_fail(c, e, "work model counts");
+    }
+    auto model_of = [&](const ClassKey& k, const unsigned long long* n4) {
+      const ClassKey rev{k.lc, k.ld, k.la, k.lb, k.Kk, k.Kb, 0};
+      double f = 0.0;
+      for (int x = 0; x < 2; ++x)
+        for (int y = 0; y < 2; ++y) {
+          const std::array<int, 3> bra{x ? k.lb : k.la, x ? k.la : k.lb, k.Kb}, ket{y ? k.ld : k.lc, y ? k.lc : k.ld, k.Kk};
+          f += model_flops_class(bra >= ket ? k : rev) * (double)n4[2 * x + y];
+        }
+      return f;
+    };
     // one launch descriptor per non-empty bucket, plus the persistent work items
     std::vector<WorkItem> items;
     std::vector<double> cost;
@@ -2289,7 +2317,7 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
         a.mol_nao = X->molnao;
         X->launches.push_back(a);
         X->lkey.push_back(key);
-        X->lflops.push_back(model_flops_class(key) * (double)counts[b]);
+        X->lflops.push_back(model_of(key, ocounts.data() + 4 * b));
         X->model_flops += X->lflops.back();
         // persistent shape: the class's own team size T, as many teams as fit the block's
         // threads and kPersistSmem of shared memory (two blocks per SM), in whole warps (the
@@ -2340,7 +2368,7 @@ mdx_status mdx_xbatch_create(mdx_ctx* c, int32_t n_mol, const mdx_basis* bases, 
           item_reg.push_back(reg_class);
         }
         X->is_reg.push_back(reg_class);
-        X->order.emplace_back(X->lflops.back(), (int32_t)(X->launches.size() - 1));
+        X->order.emplace_back(model_flops_class(key) * (double)counts[b], (int32_t)(X->launches.size() - 1));
       }
     std::stable_sort(X->order.begin(), X->order.end(),
                      [](const std::pair<double, int32_t>& x, const std::pair<double, int32_t>& y) { return x.first > y.first; });

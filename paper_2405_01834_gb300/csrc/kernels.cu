@@ -1347,6 +1347,38 @@ __global__ void __launch_bounds__(256) k_screen(const ScreenArgs a, bool fill) {
   }
 }
 
+// Quartets of each bucket by the order of the shells in their pairs: counts[4 b + 2 x + y], x and y the flags (bit 0 of
+// class_flag, the class above it) of the bra and the ket pair. A thread takes a run of the list, which is sorted by
+// bucket, so that it adds to few counters.
+constexpr int kOrderRun = 64;
+__global__ void k_order_counts(const int2* __restrict__ quart, int64_t nq, const int32_t* __restrict__ class_flag,
+                               unsigned long long* __restrict__ counts) {
+  const int64_t q0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kOrderRun;
+  int64_t cur = -1;
+  unsigned long long n = 0;
+  for (int64_t q = q0; q < q0 + kOrderRun && q < nq; ++q) {
+    const int2 pq = quart[q];
+    const int x = class_flag[pq.x], y = class_flag[pq.y];
+    const int64_t cp = x >> 1, at = (cp * (cp + 1) / 2 + (y >> 1)) * 4 + 2 * (x & 1) + (y & 1);
+    if (at != cur) {
+      if (n) atomicAdd(counts + cur, n);
+      cur = at;
+      n = 0;
+    }
+    ++n;
+  }
+  if (n) atomicAdd(counts + cur, n);
+}
+
+cudaError_t launch_order_counts(const int2* quart, int64_t nq, const int32_t* class_flag, unsigned long long* counts,
+                                cudaStream_t s) {
+  if (nq <= 0) return cudaSuccess;
+  const int64_t per = 128 * (int64_t)kOrderRun, grid = (nq + per - 1) / per;
+  if (grid > 0x7fffffff) return cudaErrorInvalidValue;
+  k_order_counts<<<(unsigned)grid, 128, 0, s>>>(quart, nq, class_flag, counts);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_screen(const ScreenArgs& a, bool fill, cudaStream_t s) {
   if (a.npairs <= 0) return cudaSuccess;
   if (a.npairs > 0x7fffffff) return cudaErrorInvalidValue;

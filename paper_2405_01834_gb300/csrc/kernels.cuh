@@ -155,6 +155,10 @@ struct ScreenArgs {
   int2* out;                   // fill pass: (p, q) per surviving quartet
 };
 cudaError_t launch_screen(const ScreenArgs& a, bool fill, cudaStream_t s);
+// Quartets per bucket and order of the shells in the two pairs: counts[4 b + 2 x + y] += 1 for bucket
+// b = cp (cp + 1) / 2 + cq, class_flag[pair] = 2 class + flag; counts zeroed by the caller.
+cudaError_t launch_order_counts(const int2* quart, int64_t nq, const int32_t* class_flag, unsigned long long* counts,
+                                cudaStream_t s);
 // out[2k], out[2k+1] = orig[qp[k].x], orig[qp[k].y] (sorted pair indices back to caller indices)
 cudaError_t launch_map_pairs(const int2* qp, int64_t n, const int64_t* orig, int32_t* out, cudaStream_t s);
 cudaError_t launch_symmetrize(double* K, int32_t nao, cudaStream_t s);
