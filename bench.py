@@ -954,6 +954,7 @@ def main():
     peak_gflops = max(probe.values())
     total_flops = sum(model_flops(l, len(q)) for l, _, q, _ in prepared)
     total_exec = sum(2.0 * bt.exec_fma for *_, batches in prepared for bt in batches)
+    total_instr = sum(fp64_instr(bt) for *_, batches in prepared for bt in batches)
     value = whole_job_rate(total_flops, world, ms_step) * 1e-9
     per_class = {}
     dom_l, dom_ms = None, -1.0
@@ -965,13 +966,17 @@ def main():
             "quartets": len(q), "ms": round(ms, 3), "quartets_per_s": round(len(q) / (ms * 1e-3), 1),
             "exec_gflops": round(ex / (ms * 1e-3) * 1e-9, 2),
             "exec_frac_of_peak": round(ex / (ms * 1e-3) * 1e-9 / peak_gflops, 4),
+            "fp64_pipe_frac": round(sum(2 * fp64_instr(bt) for bt in batches) / (ms * 1e-3) * 1e-9 / peak_gflops, 4),
+            "kernel": batches[0].classes()[0]["kernel"],
             "model_gflops": round(f / (ms * 1e-3) * 1e-9, 2),
             "model_over_executed_flops": round(f / ex, 2),
             "launches_per_step": 2 * len(batches)}
         if ms > dom_ms:
             dom_ms, dom_l = ms, l
-    # roofline of the dominant class's launches (pair records + quartet kernel per chunk): the FP64
-    # multiply-adds its planner counts (x2) per launch over the launch's CUDA-event time
+    # roofline of the dominant class's launches (pair records + quartet kernel per chunk): the FP64 operations
+    # that the batch counts (2 per multiply-add) per launch over the launch's CUDA-event time; beside it the share of
+    # the FP64 pipe that the issued instructions take (a multiplication holds the pipe as long as a multiply-add, so
+    # for k_rys, two instructions for three operations, the pipe bounds `frac` at 3/4)
     l = dom_l
     _, _, q, batches = next(p for p in prepared if p[0] == l)
     lm = per_launch_ms[l]
@@ -982,10 +987,14 @@ def main():
     traffic = None
     if NCU_DRAM_BYTES_PER_II_QUARTET is not None and l == 6:
         traffic = round(NCU_DRAM_BYTES_PER_II_QUARTET * len(q) / len(batches))
-    roofline = {"bound": "alu", "kernel": "%s %s" % ("k_rys" if l > 1 else "k_reg_single", CLASS_NAMES[l]), "achieved": round(achieved, 4),
+    per_launch_instr = sum(fp64_instr(bt) for bt in batches) / len(batches)
+    roofline = {"bound": "alu", "kernel": "%s %s" % (batches[0].classes()[0]["kernel"], CLASS_NAMES[l]),
+                "achieved": round(achieved, 4),
                 "peak": round(peak_gflops * 1e-3, 4), "unit": "TFLOP/s", "frac": round(achieved / (peak_gflops * 1e-3), 4),
                 "traffic": traffic, "traffic_unit": "DRAM bytes read + written per launch (ncu)",
                 "algorithmic_flops_per_launch": per_launch_exec,
+                "fp64_instructions_per_launch": per_launch_instr,
+                "fp64_pipe_frac": round(2 * per_launch_instr / (avg_launch_ms * 1e-3) * 1e-9 / peak_gflops, 4),
                 "peak_basis": "FP64, measured in this run: max of scalar DFMA %.1f and DMMA m8n8k4 %.1f GFLOP/s "
                               "(mdx_fp64_peak); derived 2 FMA/clk/SM x %d SMs x %.0f MHz = %.1f GFLOP/s" % (
                                   probe["dfma"], probe["dmma_m8n8k4"], props.multi_processor_count, sm_max,
@@ -1000,6 +1009,7 @@ def main():
             "quartets_per_s": round(whole_job_rate(sum(len(q) for _, _, q, _ in prepared), world, ms_step), 1),
             "exec_gflops": round(world * total_exec / (ms_step * 1e-3) * 1e-9, 3),
             "exec_frac_of_peak": round(total_exec / (ms_step * 1e-3) * 1e-9 / peak_gflops, 4),
+            "fp64_pipe_frac": round(2 * total_instr / (ms_step * 1e-3) * 1e-9 / peak_gflops, 4),
             "fp64_peak_gflops": {k: round(v, 1) for k, v in probe.items()},
             "per_class": per_class, "roofline": roofline, "autotune_s": tuned or None, "gpu_launches": launches,
             "gpu_launches_per_step": launches // args.steps if args.steps else 0,
@@ -1025,6 +1035,11 @@ def main():
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
+
+
+def fp64_instr(batch):
+    """FP64 instructions of one run of a prepared batch."""
+    return sum(c["n"] * c["fp64_instr"] for c in batch.classes())
 
 
 def sample_parity(prepared, kept, out, torch):

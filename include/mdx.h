@@ -203,9 +203,36 @@ mdx_status mdx_batch_eri3(mdx_ctx* ctx, const mdx_basis* aux, const mdx_basis* o
 /* Sizes of a prepared batch (host values; any pointer may be NULL): number of
  * quartets, output doubles, model FLOPs of the paper's Table 1 work model
  * adapted to contracted Cartesian shellsets, and FP64 multiply-adds the
- * engine issues. */
+ * engine issues (its floating-point operations over two: a lone
+ * multiplication of the Rys kernel counts half; the register kernels' single
+ * products of expansion coefficients, a few in a hundred, count as one). */
 mdx_status mdx_batch_info(const mdx_batch* batch, int64_t* n, int64_t* total, double* model_flops,
                           double* exec_fma);
+
+/* The launch of class i of a prepared batch (classes in the batch's order,
+ * MDX_EINVAL past the last): its angular momenta (l[1] = 0 with one_centre),
+ * primitive pairs of bra and ket, quartets, the kernel that a run takes, the
+ * lanes (register kernel) or teams (team kernel) that share one quartet, and
+ * per shellset the multiply-adds of mdx_batch_info and the FP64 instructions
+ * issued for them (what the FP64 pipe is busy with: the two differ where a
+ * kernel multiplies without adding). After mdx_batch_autotune: of the shapes
+ * it chose. */
+enum {
+  MDX_KERNEL_TEAM = 0,
+  MDX_KERNEL_REGISTER = 1,
+  MDX_KERNEL_REGISTER_SINGLE = 2,   /* uncontracted: one-warp blocks without shared memory */
+  MDX_KERNEL_RYS = 3,
+  MDX_KERNEL_TEAM_SPH = 4
+};
+typedef struct {
+  int32_t l[4];
+  int32_t K_bra, K_ket, one_centre;
+  int32_t kernel;
+  int64_t n;
+  int32_t lanes, teams;
+  double exec_fma, fp64_instr;
+} mdx_class_run;
+mdx_status mdx_batch_class(const mdx_batch* batch, int32_t i, mdx_class_run* out);
 
 /* Copy the batch's [n+1] output offsets (see mdx_eri4) to out_offsets (device). */
 mdx_status mdx_batch_offsets(mdx_ctx* ctx, const mdx_batch* batch, int64_t* out_offsets, void* stream);
@@ -442,7 +469,9 @@ mdx_status mdx_fp64_peak(int kind, int reps, double* gflops, void* stream);
  * of the resulting step programs stays inside the team workspace; a class
  * that cannot be planned returns MDX_EUNSUPPORTED.
  * exec_fma: FP64 multiply-adds the kernel issues per contracted shellset
- * (transforms, R recursion and Boys interpolation). */
+ * (transforms, R recursion and Boys interpolation), by the step programs or
+ * the register kernel's transforms. A batch may take another form of the same
+ * class (Rys kernel, kets as sums of scaled R tables): mdx_batch_class. */
 typedef struct {
   int32_t team_threads;
   int32_t teams_per_cta;

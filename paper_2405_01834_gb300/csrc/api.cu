@@ -306,6 +306,7 @@ struct mdx_batch {
   std::vector<int64_t> qorig;     // caller index of each class-sorted quartet
   double model_flops = 0.0;
   double exec_fma = 0.0;
+  double fp64_instr = 0.0;
   bool owned = true;              // device arrays belong to the batch (else: context workspace of one call)
 };
 
@@ -405,6 +406,9 @@ struct Fanout {
   int width = 1;
   double load[mdx_ctx::kAux + 1] = {};
   cudaStream_t stream(int i) const { return i == 0 ? s : c->aux[i - 1]; }
+  static int width_of(size_t launches) {
+    return 1 + (int)std::min<size_t>(mdx_ctx::kAux, launches > 0 ? launches - 1 : 0);
+  }
   static cudaError_t capture_id(cudaStream_t st, unsigned long long* id) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     *id = 0;
@@ -413,8 +417,8 @@ struct Fanout {
     return e;
   }
   cudaError_t fork(size_t launches) {
-    const int want = (int)std::min<size_t>(mdx_ctx::kAux, launches > 0 ? launches - 1 : 0);
-    width = want + 1;
+    width = width_of(launches);
+    const int want = width - 1;
     if (want == 0) return cudaSuccess;
     unsigned long long own = 0, other = 0;
     cudaError_t e = capture_id(s, &own);
@@ -459,6 +463,56 @@ double model_flops_class(const ClassKey& k, bool sph = false) {
 // FP64 multiply-adds of k_cart2sph on one shellset (every product of non-zero coefficients once).
 double cart2sph_fma(const ClassKey& k) {
   return (double)solid_nnz(k.la) * solid_nnz(k.lb) * solid_nnz(k.lc) * solid_nnz(k.ld);
+}
+
+// What a run of the batch launches for range r, per shellset: see mdx_class_run.
+mdx_class_run class_run(const mdx_batch* B, const mdx_batch::Range& r) {
+  const ClassKey& k = r.key;
+  const PlanDev& P = r.plan->d;
+  mdx_class_run o{};
+  o.l[0] = k.la; o.l[1] = k.lb; o.l[2] = k.lc; o.l[3] = k.ld;
+  o.K_bra = k.Kb;
+  o.K_ket = k.Kk;
+  o.one_centre = k.onec;
+  o.n = r.count;
+  o.lanes = o.teams = 1;
+  if (B->sph && r.splan) {
+    o.kernel = MDX_KERNEL_TEAM_SPH;
+    o.exec_fma = o.fp64_instr = r.splan->exec_fma;
+    return o;
+  }
+  if (!B->sph && P.rys) {
+    o.kernel = MDX_KERNEL_RYS;
+    o.exec_fma = r.plan->rys_fma;
+    o.fp64_instr = r.plan->rys_instr;
+    return o;
+  }
+  const int width = Fanout::width_of(B->ranges.size());
+  o.exec_fma = r.plan->exec_fma;
+  if (P.reg) {
+    const RegShape s = reg_shape(P, r.count, width, false);
+    o.kernel = s.single ? MDX_KERNEL_REGISTER_SINGLE : MDX_KERNEL_REGISTER;
+    o.lanes = s.single ? 1 : 1 << (s.split_b + s.split_k);
+    if (s.sums) o.exec_fma += k.Kb * (k.Kk * (s.sums_per_prim - r.plan->ket_fma) + s.sums_per_bra);
+  } else {
+    int nb, nk;
+    o.kernel = MDX_KERNEL_TEAM;
+    team_parts(P, r.count, width, true, &nb, &nk);
+    o.teams = nb * nk;
+  }
+  if (B->sph) o.exec_fma += cart2sph_fma(k);
+  o.fp64_instr = o.exec_fma;
+  return o;
+}
+
+// The batch's totals of what its classes run now.
+void batch_counts(mdx_batch* B) {
+  B->exec_fma = B->fp64_instr = 0.0;
+  for (const auto& r : B->ranges) {
+    const mdx_class_run o = class_run(B, r);
+    B->exec_fma += o.exec_fma * (double)o.n;
+    B->fp64_instr += o.fp64_instr * (double)o.n;
+  }
 }
 
 // Host preparation of a batch: primitive-pair jobs, class grouping, plans,
@@ -528,7 +582,6 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
     if ((st = get_plan(c, kv.first, &plan, s)) != MDX_OK) return st;
     Plan* splan = nullptr;
     int grid = 0;
-    double fma = plan->exec_fma;
     if (!sph && plan->d.rys) {
       if ((st = need_rys_table(c, s)) != MDX_OK) return st;
       int resident = 0;
@@ -537,7 +590,6 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
       rys_total = std::max<int64_t>(rys_total, (int64_t)grid * plan->d.ry_table);
       rys_stride = std::max<int64_t>(rys_stride, plan->d.ry_table);
       rys_resident = std::max(rys_resident, resident);
-      fma = plan->rys_fma;
     }
     ClassKey ks = kv.first;
     ks.store = 2;
@@ -548,7 +600,6 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
       cudaError_t e = sph_grid(splan->d, cnt, &grid);
       if (e != cudaSuccess) return cuda_fail(c, e, "solid-harmonic launch shape");
       xg_total = std::max<int64_t>(xg_total, (int64_t)grid * splan->d.teams_per_cta * splan->d.xg_doubles);
-      fma = splan->exec_fma;
     }
     if (sph) {
       cqoff.resize(qp_sorted.size(), 0);
@@ -559,15 +610,14 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
           cqoff[i] = cart_total;
           cart_total += nct;
         }
-        fma += cart2sph_fma(k);
       }
     }
     B->ranges.push_back({plan, b, cnt, kv.first, splan, grid});
     const double model = model_flops_class(kv.first, sph) * (double)cnt;
     B->order.emplace_back(model, (int32_t)B->ranges.size() - 1);
     B->model_flops += model;
-    B->exec_fma += fma * (double)cnt;
   }
+  batch_counts(B.get());
   std::stable_sort(B->order.begin(), B->order.end(),
                    [](const std::pair<double, int32_t>& x, const std::pair<double, int32_t>& y) { return x.first > y.first; });
   B->njobs = (int64_t)jobs.size();
@@ -1031,6 +1081,12 @@ mdx_status mdx_batch_info(const mdx_batch* b, int64_t* n, int64_t* total, double
   return MDX_OK;
 }
 
+mdx_status mdx_batch_class(const mdx_batch* b, int32_t i, mdx_class_run* out) {
+  if (!b || !out || i < 0 || i >= (int32_t)b->ranges.size()) return MDX_EINVAL;
+  *out = class_run(b, b->ranges[i]);
+  return MDX_OK;
+}
+
 mdx_status mdx_batch_offsets(mdx_ctx* c, const mdx_batch* b, int64_t* out_offsets, void* stream) {
   if (!c || !b || !out_offsets) return MDX_EINVAL;
   cudaSetDevice(c->device);
@@ -1289,9 +1345,6 @@ mdx_status autotune_sph(mdx_ctx* c, mdx_batch* b, double* out, int64_t max_trial
       b->nxg = need;
     }
     c->tuned[k2] = best;
-    // the batch's executed-FMA count follows the route and shape the class runs now
-    const double old_fma = r.splan ? r.splan->exec_fma : r.plan->exec_fma + cart2sph_fma(r.key);
-    b->exec_fma += (best_plan->exec_fma - old_fma) * (double)r.count;
     auto it = c->plans.find(k2);
     if (it != c->plans.end()) c->retired.push_back(std::move(it->second));
     r.splan = best_plan.get();
@@ -1302,6 +1355,7 @@ mdx_status autotune_sph(mdx_ctx* c, mdx_batch* b, double* out, int64_t max_trial
   for (auto& r : b->ranges)
     if (r.splan && (int64_t)r.grid * r.splan->d.teams_per_cta * r.splan->d.xg_doubles > b->nxg)
       return done(fail(c, MDX_EINVAL, "solid-harmonic staging area smaller than a class needs"));
+  batch_counts(b);   // of the routes and shapes the classes run now
   done(MDX_OK);
   return check_device_error(c, s);
 }
@@ -1410,13 +1464,12 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
     }
     if (!best_plan) continue;
     c->tuned[r.key] = best;
-    b->exec_fma += (best_plan->exec_fma - (r.plan->d.rys ? r.plan->rys_fma : r.plan->exec_fma)) *
-                   (double)r.count;   // the shape it runs now
     auto it = c->plans.find(r.key);
     if (it != c->plans.end()) c->retired.push_back(std::move(it->second));
     r.plan = best_plan.get();
     c->plans[r.key] = std::move(best_plan);
   }
+  batch_counts(b);   // of the shapes the classes run now
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   return check_device_error(c, s);

@@ -1183,20 +1183,18 @@ static const RegPart kRegParts[] = {launch_reg_part00, launch_reg_part01, launch
 // Measured: one-shot 4-center call on 2 atoms 5.17 -> 2.04 ms ([dd|dd] K = 81: one team's 0.85 ms chain in
 // 8 parts); exchange of 5 atoms 90 -> 77 ms and 8-molecule batched exchange 73 -> 63 ms, where without the
 // share of the SMs the repeated work made the gradient of 3 atoms slower (162 -> 173 ms; with it 149).
-static void team_parts(const QuartetLaunch& a, int* nb, int* nk) {
-  const PlanDev& P = a.plan;
+void team_parts(const PlanDev& P, int64_t nq, int concurrent, bool store, int* nb, int* nk) {
   *nb = *nk = 1;
   if (P.Kb * P.Kk == 1 || !P.has_out) return;
-  const bool store = !a.D && !a.grad;
   const int64_t cta = (int64_t)P.teams_per_cta * P.team_doubles * 8 + 1024, block = P.teams_per_cta * P.T;
   const int64_t fit = std::min<int64_t>(228 * 1024 / cta, std::max<int64_t>(1, 512 / block));
-  const double sat = 152.0 * (double)std::max<int64_t>(1, fit) * P.teams_per_cta / std::max(1, a.concurrent);
+  const double sat = 152.0 * (double)std::max<int64_t>(1, fit) * P.teams_per_cta / std::max(1, concurrent);
   const double ck = P.cost_k, cb = P.cost_b, ce = store ? 0.2 * P.cost_b : P.cost_b;
   double best = 1e300;
   for (int b = 1; b <= std::min(P.Kb, store ? 8 : 64); ++b)
     for (int k = 1; k <= std::min(P.Kk, (store ? 8 : 64) / b); ++k) {
       const double chain = (double)((P.Kb + b - 1) / b) * ((double)((P.Kk + k - 1) / k) * ck + cb) + ce;
-      const double t = chain * std::max(1.0, (double)a.nq * b * k / sat);
+      const double t = chain * std::max(1.0, (double)nq * b * k / sat);
       if (t < 0.95 * best) { best = t; *nb = b; *nk = k; }
     }
 }
@@ -1215,7 +1213,7 @@ cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s) {
     }
   }
   QuartetLaunch b = a;
-  team_parts(a, &b.part_b, &b.part_k);
+  team_parts(P, a.nq, a.concurrent, !a.D && !a.grad, &b.part_b, &b.part_k);
   const int parts = b.part_b * b.part_k;
   const int64_t grid = (a.nq + P.teams_per_cta - 1) / P.teams_per_cta * parts;
   const int block = P.teams_per_cta * P.T;

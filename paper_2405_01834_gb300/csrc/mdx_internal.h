@@ -213,7 +213,9 @@ struct Plan {
   std::vector<uint16_t> colmap;
   std::vector<uint16_t> colinv;
   double exec_fma = 0;     // FMAs executed per primitive-quartet pass (for reports)
-  double rys_fma = 0;      // FP64 instructions of the Rys kernel per shellset (d.rys)
+  double ket_fma = 0;      // of it, the register kernel's ket transform of one primitive quartet
+  double rys_fma = 0;      // the Rys kernel (d.rys) per shellset: multiply-adds, a lone multiplication as half,
+  double rys_instr = 0;    // and FP64 instructions
   void* dev_blob = nullptr;
 };
 

@@ -272,12 +272,15 @@ static void plan_rys(Plan& plan) {
       for (int y = 0; y <= l2; ++y) t += x + y + 1;
     return t;
   };
-  plan.rys_fma = 2.0 * n * P.Nb * P.Nk + 3.0 * n * (terms(P.la, P.lb) * ncd1 + (P.Lb + 1) * terms(P.lc, P.ld)) +
-                 3.0 * n * 2.0 * P.L + 2.0 * n * kRysTerms;
-  // Both are bound by the FP64 pipe, so the count decides. Measured (team kernel -> this one, same grids):
+  // per integral and node a product and a multiply-add: two instructions, three operations
+  const double tables = 3.0 * n * (terms(P.la, P.lb) * ncd1 + (P.Lb + 1) * terms(P.lc, P.ld)) + 3.0 * n * 2.0 * P.L +
+                        2.0 * n * kRysTerms;
+  plan.rys_fma = 1.5 * n * P.Nb * P.Nk + tables;
+  plan.rys_instr = 2.0 * n * P.Nb * P.Nk + tables;
+  // Both are bound by the FP64 pipe, so the instruction count decides. Measured (team kernel -> this one, same grids):
   // [61|00] 627 -> 432 us, [22|22] 2.08 -> 1.42 ms, [ff|ff] 4.02 -> 2.40 ms, [ii|ii] 27.5 -> 14.8 ms, 3-center
   // [6|10] 476 -> 378 us, [3|33] 6.48 -> 1.62 ms, [6|66] 11.6 -> 4.63 ms; no class of L >= 7 was slower.
-  if (n > kRysMax || plan.rys_fma > 0.97 * plan.exec_fma) return;
+  if (n > kRysMax || plan.rys_instr > 0.97 * plan.exec_fma) return;
   // records, nodes and weights, one-dimensional functions, index words (and one for the block's table area)
   const int fixed = P.recb + P.reck + 2 * n + 3 * (P.L + 1) * n + ((P.Nb + P.Nk + nab1 + ncd1 + 1) / 2 + 1);
   auto doubles = [&](int cw, int rows) {
@@ -704,6 +707,7 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
         bra += eprod(nx, ny, nz) + (double)P.Nk * nx * ny * nz;
       }
     plan.exec_fma = key.Kb * key.Kk * (fma_r + 8.0 * (P.L + 1) + ket) + key.Kb * bra;
+    plan.ket_fma = ket;
   }
 
   if (!validate_plan(plan, err)) return false;

@@ -731,6 +731,18 @@ inline void split_of(int64_t nq, int concurrent, int Kb, int Kk, double ck, doub
     }
 }
 
+// The cost arguments of split_of for a class.
+struct SplitCost {
+  double ck, cb, cr;
+};
+constexpr SplitCost split_cost(int la, int lb, int lc, int ld) {
+  const double body = reg_body_size(la, lb, lc, ld), ket = reg_body_size(la, lb, lc, ld, false);
+  return {ket + 8.0 * (la + lb + lc + ld + 1) + 80.0, body - ket,
+          (double)(ncart(la) * ncart(lb) * ncart(lc) * ncart(ld))};
+}
+// Ket primitives per lane decide between the instance that sums R tables and the one that does not.
+inline bool runs_sums(int Kk, int split_k) { return ((Kk + (1 << split_k) - 1) >> split_k) >= kKetSumsMin; }
+
 // Uncontracted shellsets of the classes below: one warp per block, one thread per quartet, everything in registers. The
 // columns [p|cd] are formed one at a time and go through the bra transform at once, so that neither [p|cd] nor the
 // shellset is ever whole; the products of the bra's E tables are formed once. The shared-memory variant holds [p|cd]
@@ -864,8 +876,7 @@ cudaError_t launch_reg_epilogue(const QuartetLaunch& a, unsigned grid, cudaStrea
       return cudaGetLastError();
     }
   }
-  const int per = (a.plan.Kk + (1 << a.split_k) - 1) >> a.split_k;   // ket primitives per lane
-  if (KS && per >= kKetSumsMin) sums<<<grid, bs, shm_s, s>>>(a);
+  if (KS && runs_sums(a.plan.Kk, a.split_k)) sums<<<grid, bs, shm_s, s>>>(a);
   else plain<<<grid, bs, shm, s>>>(a);
   return cudaGetLastError();
 }
@@ -874,11 +885,9 @@ template <int LA, int LB, int LC, int LD>
 cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
   constexpr bool XS = !reg_eligible(LA, LB, LC, LD);
   constexpr int bs = XS ? kXsBlock : 128;
-  constexpr int Nk = ncart(LC) * ncart(LD);
   QuartetLaunch a = a0;
-  constexpr double ck = reg_body_size(LA, LB, LC, LD, false) + 8.0 * (LA + LB + LC + LD + 1) + 80.0;
-  constexpr double cb = reg_body_size(LA, LB, LC, LD) - reg_body_size(LA, LB, LC, LD, false);
-  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, ck, cb, (double)ncart(LA) * ncart(LB) * Nk, &a.split_b, &a.split_k);
+  constexpr SplitCost sc = split_cost(LA, LB, LC, LD);
+  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, sc.ck, sc.cb, sc.cr, &a.split_b, &a.split_k);
   const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   return a.D ? launch_reg_epilogue<LA, LB, LC, LD, true>(a, (unsigned)grid, s)

@@ -35,6 +35,13 @@ class PlanStats(ctypes.Structure):
                 ("register_kernel", ctypes.c_int32), ("pad", ctypes.c_int32)]
 
 
+class ClassRun(ctypes.Structure):
+    _fields_ = [("l", ctypes.c_int32 * 4), ("K_bra", ctypes.c_int32), ("K_ket", ctypes.c_int32),
+                ("one_centre", ctypes.c_int32), ("kernel", ctypes.c_int32), ("n", ctypes.c_int64),
+                ("lanes", ctypes.c_int32), ("teams", ctypes.c_int32), ("exec_fma", ctypes.c_double),
+                ("fp64_instr", ctypes.c_double)]
+
+
 def plan_info(la, lb, lc, ld, Kb=1, Kk=1, one_centre=False) -> PlanStats:
     """Team shape and executed FP64 FMA count per shellset of a class (host planner, no GPU)."""
     lib = load()
@@ -147,6 +154,8 @@ def load(build_if_missing: bool = True):
     lib.mdx_exchange_screen.restype = I32
     lib.mdx_last_quartet_count.argtypes = [P]
     lib.mdx_last_quartet_count.restype = I64
+    lib.mdx_batch_class.argtypes = [P, I32, ctypes.POINTER(ClassRun)]
+    lib.mdx_batch_class.restype = I32
     lib.mdx_eri4_noalloc.argtypes = [ctypes.POINTER(_Basis), P, I64, P, I64, P, P]
     lib.mdx_eri4_noalloc.restype = I32
     lib.mdx_xbatch_create.argtypes = [P, I32, P, P, P, ctypes.c_double, ctypes.POINTER(ctypes.c_void_p), P]
@@ -447,6 +456,20 @@ class Batch:
         self.eng._check(self.eng.lib.mdx_batch_info(self.h, ctypes.byref(n), ctypes.byref(tot), ctypes.byref(mf),
                                                     ctypes.byref(ef)), "mdx_batch_info")
         self.n, self.total, self.model_flops, self.exec_fma = n.value, tot.value, mf.value, ef.value
+
+    KERNELS = ("k_quartets", "k_reg", "k_reg_single", "k_rys", "k_quartets_sph")
+
+    def classes(self):
+        """What a run launches, class by class (see mdx_batch_class), with the kernel's name."""
+        out, i = [], 0
+        while True:
+            r = ClassRun()
+            if self.eng.lib.mdx_batch_class(self.h, i, ctypes.byref(r)) != 0:
+                return out
+            out.append({"l": tuple(r.l), "K": (r.K_bra, r.K_ket), "one_centre": bool(r.one_centre), "n": r.n,
+                        "kernel": self.KERNELS[r.kernel], "lanes": r.lanes, "teams": r.teams,
+                        "exec_fma": r.exec_fma, "fp64_instr": r.fp64_instr})
+            i += 1
 
     def offsets(self) -> torch.Tensor:
         o = torch.empty(self.n + 1, dtype=torch.int64, device="cuda")
