@@ -40,10 +40,8 @@ UNIT = "GFLOP/s (Table-1 model FLOPs)"
 # peak that is reported beside the measured one
 FP64_FLOP_PER_CLK_SM = 4.0
 CHUNK_BYTES = 2 << 30
-# DRAM bytes (read + write) per [ii|ii] quartet of one k_rys launch of the benchmark (456 quartets):
-# ncu --nvtx --nvtx-include "mdx_batch_run/" -k regex:k_rys -c 1 --metrics
-# dram__bytes_read.sum,dram__bytes_write.sum on `bench.py --classes 6 --n-bra 24 --n-ket 19 --steps 1
-# --warmup 3 --no-cpu --no-e2e`: 1,000,510,464 B read + 2,647,006,464 B written
+# DRAM bytes (read + write) per [ii|ii] quartet of one k_rys launch of the benchmark (456 quartets), from the
+# capture whose command is in profiles/k_rys_ii_bench_launch.md: 1,000,510,464 B read + 2,647,006,464 B written
 NCU_DRAM_BYTES_PER_II_QUARTET = (1000510464 + 2647006464) / 456
 
 
