@@ -1228,6 +1228,8 @@ mdx_status autotune_sph(mdx_ctx* c, mdx_batch* b, double* out, int64_t max_trial
       QuartetLaunch a{};
       a.plan = r.plan->d;
       a.nq = nq;
+      a.share_nq = r.count;
+      a.concurrent = Fanout::width_of(b->ranges.size());
       a.qpairs = b->qp + r.begin;
       a.qout = b->cqoff + r.begin;
       a.pair_rec = b->pair_rec;
@@ -1432,6 +1434,8 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
       QuartetLaunch a{};
       a.plan = p->d;
       a.nq = std::min(r.count, max_trial);
+      a.share_nq = r.count;   // lanes and teams per quartet as in a run of the batch
+      a.concurrent = Fanout::width_of(b->ranges.size());
       a.qpairs = b->qp + r.begin;
       a.qout = b->qoff + r.begin;
       a.pair_rec = b->pair_rec;
@@ -2563,6 +2567,8 @@ mdx_status mdx_xbatch_autotune(mdx_ctx* c, mdx_xbatch* xb, int64_t max_trial, vo
       QuartetLaunch a = a0;
       a.plan = p->d;
       a.nq = std::min(a0.nq, max_trial);
+      a.share_nq = a0.nq;   // lanes and teams per quartet as in a run of the batch
+      a.concurrent = Fanout::width_of(xb->order.size());
       float ms = 1e30f;
       for (int rep = 0; rep < 2; ++rep) {
         cudaEventRecord(e0, s);

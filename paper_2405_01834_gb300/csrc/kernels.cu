@@ -1213,7 +1213,7 @@ cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s) {
     }
   }
   QuartetLaunch b = a;
-  team_parts(P, a.nq, a.concurrent, !a.D && !a.grad, &b.part_b, &b.part_k);
+  team_parts(P, a.share_nq ? a.share_nq : a.nq, a.concurrent, !a.D && !a.grad, &b.part_b, &b.part_k);
   const int parts = b.part_b * b.part_k;
   const int64_t grid = (a.nq + P.teams_per_cta - 1) / P.teams_per_cta * parts;
   const int block = P.teams_per_cta * P.T;

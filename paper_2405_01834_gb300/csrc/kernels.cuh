@@ -70,6 +70,8 @@ struct QuartetLaunch {
   double* const* mol_K;
   const int32_t* mol_nao;
   int32_t concurrent;        // launches that can run side by side with it, itself included (0: alone)
+  int64_t share_nq;          // quartets that the lanes and teams per quartet are chosen for (0: nq; an autotuner's
+                             // trial runs some of a launch's quartets the way the launch runs them)
   // register kernel: 2^(split_b + split_k) lanes share a quartet's primitives (set by its launcher)
   int32_t split_b, split_k;
   // team kernel: part_b x part_k teams share a quartet's primitive pairs (set by launch_quartets)

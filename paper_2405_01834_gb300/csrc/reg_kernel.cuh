@@ -887,7 +887,8 @@ cudaError_t launch_reg_class(const QuartetLaunch& a0, cudaStream_t s) {
   constexpr int bs = XS ? kXsBlock : 128;
   QuartetLaunch a = a0;
   constexpr SplitCost sc = split_cost(LA, LB, LC, LD);
-  split_of(a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, sc.ck, sc.cb, sc.cr, &a.split_b, &a.split_k);
+  split_of(a.share_nq ? a.share_nq : a.nq, a.concurrent, a.plan.Kb, a.plan.Kk, sc.ck, sc.cb, sc.cr, &a.split_b,
+           &a.split_k);
   const int64_t grid = ((a.nq << (a.split_b + a.split_k)) + bs - 1) / bs;
   if (grid > 0x7fffffff) return cudaErrorInvalidValue;
   return a.D ? launch_reg_epilogue<LA, LB, LC, LD, true>(a, (unsigned)grid, s)
