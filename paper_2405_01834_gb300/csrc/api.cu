@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <map>
 #include <memory>
 #include <string>
@@ -168,7 +169,13 @@ mdx_status get_plan(mdx_ctx* c, const ClassKey& k, Plan** out, cudaStream_t s) {
 // non-blocking streams do not wait for: copied on `s`, and waited for, so that every later launch comes after it)
 mdx_status need_rys_table(mdx_ctx* c, cudaStream_t s) {
   if (c->d_rys) return MDX_OK;
-  const std::vector<double>& tab = rys_table();
+  const std::vector<double>* host = nullptr;
+  try {
+    host = &rys_table();
+  } catch (const std::exception&) {
+    return fail(c, MDX_ENOMEM, "Rys table: out of host memory");
+  }
+  const std::vector<double>& tab = *host;
   double* p = nullptr;
   if (cudaMalloc((void**)&p, tab.size() * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();

@@ -14,6 +14,7 @@
 // the part of the measure beyond t = 1 is exp(-100).
 #include <algorithm>
 #include <cmath>
+#include <exception>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -210,8 +211,15 @@ std::vector<double> build() {
   std::vector<double> tab((size_t)rys_offset(N + 1), 0.0);
   const Legendre gl;
   const int nt = std::max(1, std::min(16, (int)std::thread::hardware_concurrency()));
-  auto work = [&](int t0) {
-    for (int iv = t0; iv < kRysIntervals; iv += nt) interval(gl, iv, tab.data());
+  std::exception_ptr failed;   // the first exception (memory) of any thread, for the caller
+  std::mutex mu;
+  auto work = [&](int t0) noexcept {
+    try {
+      for (int iv = t0; iv < kRysIntervals; iv += nt) interval(gl, iv, tab.data());
+    } catch (...) {
+      const std::lock_guard<std::mutex> lock(mu);
+      if (!failed) failed = std::current_exception();
+    }
   };
   std::vector<std::thread> th;
   try {
@@ -222,6 +230,7 @@ std::vector<double> build() {
   const int started = (int)th.size() + 1;
   for (auto& t : th) t.join();
   for (int t = started; t < nt; ++t) work(t);   // threads that could not be started
+  if (failed) std::rethrow_exception(failed);
   // x^(-1/2) exp(-x): al_k = 2k + 1/2, be_k = k (k - 1/2), be_0 = sqrt(pi)
   dd al[N + 1], be[N + 1];
   for (int k = 0; k <= N; ++k) {
@@ -243,7 +252,7 @@ std::vector<double> build() {
 }  // namespace
 
 const std::vector<double>& rys_table() {
-  static const std::vector<double> tab = build();   // once per process, on first use
+  static const std::vector<double> tab = build();   // once per process, on first use (again after an exception)
   return tab;
 }
 
