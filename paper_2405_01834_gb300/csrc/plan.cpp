@@ -793,7 +793,9 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
         p2.exec_fma + 2.0 * r_alt < 0.9 * (plan.exec_fma + 2.0 * r_cur))
       plan = std::move(p2);
   }
-  if (key.store == 1 && key.Kb * key.Kk == 1 && !P.reg && cfg.variant == 0 && cfg.T == 0 && cfg.rys != 0)
+  // (a team size or budget that a caller asks for means the team kernel)
+  const bool team_asked = cfg.variant != 0 || cfg.T != 0 || cfg.budget != PlanConfig{}.budget;
+  if (key.store == 1 && key.Kb * key.Kk == 1 && !P.reg && !team_asked && cfg.rys != 0)
     plan_rys(plan);
   return true;
 }
