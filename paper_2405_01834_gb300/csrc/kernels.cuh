@@ -109,14 +109,13 @@ const void* persistent_kernel_ptr();
 cudaError_t launch_quartets(const QuartetLaunch& a, cudaStream_t s);
 // What launch_quartets chooses for nq quartets of a plan that can run beside concurrent - 1 other launches: the register
 // kernel's lanes per quartet (2^(split_b + split_k)) and instance, with the FP64 instructions of its sums of
-// scaled R tables per primitive quartet and per bra primitive; the team kernel's teams per quartet.
+// scaled R tables per primitive quartet and per bra primitive. (The team kernel's teams per quartet: team_parts.)
 struct RegShape {
   int split_b, split_k;
   bool single, sums;
   int sums_per_prim, sums_per_bra;
 };
 RegShape reg_shape(const PlanDev& P, int64_t nq, int concurrent, bool digest);
-void team_parts(const PlanDev& P, int64_t nq, int concurrent, bool store, int* nb, int* nk);
 // Solid-harmonic shellsets (plan.sph, store at a.out + a.qout[q]): `grid` CTAs loop over the quartets;
 // sph_grid gives the grid for nq quartets (resident CTAs at most), and a.sph_scratch must hold
 // grid * teams_per_cta * xg_doubles doubles.

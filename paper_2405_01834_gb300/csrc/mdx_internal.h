@@ -247,6 +247,10 @@ void build_rlevel_programs(std::vector<uint32_t>& prog, std::vector<int32_t>& of
 // Builds the plan of a class for the given shape.
 bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::string& err);
 
+// Teams of the team kernel that share a quartet's primitive pairs (nb x nk) in a launch of nq quartets that can run beside
+// concurrent - 1 others; store: the shellsets are stored (else digested or contracted).
+void team_parts(const PlanDev& P, int64_t nq, int concurrent, bool store, int* nb, int* nk);
+
 }  // namespace mdx
 
 namespace mdx {

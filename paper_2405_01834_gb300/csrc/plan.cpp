@@ -800,4 +800,29 @@ bool build_plan(const ClassKey& key, const PlanConfig& cfg, Plan& plan, std::str
   return true;
 }
 
+// How many teams share a quartet's bra and ket primitive pairs. A launch of few quartets of a contracted
+// class is bound by one team's chain of barrier-separated steps over its primitive quartets (about 10 us each
+// at L = 7), so its time is taken as the chain's, times the number of rounds in which the launch's teams
+// exceed those that the SMs hold with the FP64 pipe kept busy (its share of them where several launches run
+// side by side). A split over the ket pairs repeats the bra steps, and every split the epilogue. Teams that
+// store their shellset add it up inside a cluster (portable size: 8 blocks) and need the OUT region.
+// Measured: one-shot 4-center call on 2 atoms 5.17 -> 2.04 ms ([dd|dd] K = 81: one team's 0.85 ms chain in
+// 8 parts); exchange of 5 atoms 90 -> 77 ms and 8-molecule batched exchange 73 -> 63 ms, where without the
+// share of the SMs the repeated work made the gradient of 3 atoms slower (162 -> 173 ms; with it 149).
+void team_parts(const PlanDev& P, int64_t nq, int concurrent, bool store, int* nb, int* nk) {
+  *nb = *nk = 1;
+  if (P.Kb * P.Kk == 1 || !P.has_out) return;
+  const int64_t cta = (int64_t)P.teams_per_cta * P.team_doubles * 8 + 1024, block = P.teams_per_cta * P.T;
+  const int64_t fit = std::min<int64_t>(228 * 1024 / cta, std::max<int64_t>(1, 512 / block));
+  const double sat = 152.0 * (double)std::max<int64_t>(1, fit) * P.teams_per_cta / std::max(1, concurrent);
+  const double ck = P.cost_k, cb = P.cost_b, ce = store ? 0.2 * P.cost_b : P.cost_b;
+  double best = 1e300;
+  for (int b = 1; b <= std::min(P.Kb, store ? 8 : 64); ++b)
+    for (int k = 1; k <= std::min(P.Kk, (store ? 8 : 64) / b); ++k) {
+      const double chain = (double)((P.Kb + b - 1) / b) * ((double)((P.Kk + k - 1) / k) * ck + cb) + ce;
+      const double t = chain * std::max(1.0, (double)nq * b * k / sat);
+      if (t < 0.95 * best) { best = t; *nb = b; *nk = k; }
+    }
+}
+
 }  // namespace mdx
