@@ -73,8 +73,12 @@ __global__ void k_pair_records(BasisDev b0, BasisDev b1, const PrimPairJob* __re
   const double ip = 1.0 / p;
   const double inv2p = 0.5 * ip;
   double P[3], ab2 = 0.0;
+  // P = A exactly where both shells share the coordinate (always with a one-centre bra): the rounding of the quotient would
+  // give P - A of an ulp of A, and the tables' entries that vanish by parity with it (the step programs of a
+  // one-centre bra skip them, the Rys and register kernels read them): [3|22] with its shells 10 bohr apart was
+  // off by 5e-14 of its largest integral, 5e-16 now
   for (int k = 0; k < 3; ++k) {
-    P[k] = (za * A[k] + zb * Bc[k]) * ip;
+    P[k] = A[k] == Bc[k] ? A[k] : (za * A[k] + zb * Bc[k]) * ip;
     const double d = A[k] - Bc[k];
     ab2 += d * d;
   }
