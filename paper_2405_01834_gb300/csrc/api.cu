@@ -312,8 +312,6 @@ struct mdx_batch {
   std::vector<std::pair<double, int32_t>> order;   // (model FLOPs, range), heaviest first: launch order
   std::vector<int64_t> qorig;     // caller index of each class-sorted quartet
   double model_flops = 0.0;
-  double exec_fma = 0.0;
-  double fp64_instr = 0.0;
   bool owned = true;              // device arrays belong to the batch (else: context workspace of one call)
 };
 
@@ -512,16 +510,6 @@ mdx_class_run class_run(const mdx_batch* B, const mdx_batch::Range& r) {
   return o;
 }
 
-// The batch's totals of what its classes run now.
-void batch_counts(mdx_batch* B) {
-  B->exec_fma = B->fp64_instr = 0.0;
-  for (const auto& r : B->ranges) {
-    const mdx_class_run o = class_run(B, r);
-    B->exec_fma += o.exec_fma * (double)o.n;
-    B->fp64_instr += o.fp64_instr * (double)o.n;
-  }
-}
-
 // Host preparation of a batch: primitive-pair jobs, class grouping, plans,
 // uploads. Synchronises `s` before returning (host vectors go out of scope).
 // call_ws: the device arrays live in context workspace (one-shot calls: no
@@ -624,7 +612,6 @@ mdx_status batch_prepare(mdx_ctx* c, const mdx_basis* b0, const mdx_basis* b1, c
     B->order.emplace_back(model, (int32_t)B->ranges.size() - 1);
     B->model_flops += model;
   }
-  batch_counts(B.get());
   std::stable_sort(B->order.begin(), B->order.end(),
                    [](const std::pair<double, int32_t>& x, const std::pair<double, int32_t>& y) { return x.first > y.first; });
   B->njobs = (int64_t)jobs.size();
@@ -1084,7 +1071,10 @@ mdx_status mdx_batch_info(const mdx_batch* b, int64_t* n, int64_t* total, double
   if (n) *n = b->n;
   if (total) *total = b->total;
   if (model_flops) *model_flops = b->model_flops;
-  if (exec_fma) *exec_fma = b->exec_fma;
+  if (exec_fma) {   // of what the classes run now
+    *exec_fma = 0.0;
+    for (const auto& r : b->ranges) *exec_fma += class_run(b, r).exec_fma * (double)r.count;
+  }
   return MDX_OK;
 }
 
@@ -1364,7 +1354,6 @@ mdx_status autotune_sph(mdx_ctx* c, mdx_batch* b, double* out, int64_t max_trial
   for (auto& r : b->ranges)
     if (r.splan && (int64_t)r.grid * r.splan->d.teams_per_cta * r.splan->d.xg_doubles > b->nxg)
       return done(fail(c, MDX_EINVAL, "solid-harmonic staging area smaller than a class needs"));
-  batch_counts(b);   // of the routes and shapes the classes run now
   done(MDX_OK);
   return check_device_error(c, s);
 }
@@ -1480,7 +1469,6 @@ mdx_status mdx_batch_autotune(mdx_ctx* c, mdx_batch* b, double* out, int64_t out
     r.plan = best_plan.get();
     c->plans[r.key] = std::move(best_plan);
   }
-  batch_counts(b);   // of the shapes the classes run now
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   return check_device_error(c, s);
