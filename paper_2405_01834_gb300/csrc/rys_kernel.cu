@@ -56,7 +56,11 @@ struct Rule {
   static constexpr int64_t first = rys_offset(NR);
 };
 
-template <int NR>
+// AREAS: the tables live in global memory, in a free one of a.rys_areas areas. An instance of its own: one that also serves
+// the classes with tables in shared memory (and the one-shot calls, whose block b uses area b) costs the smallest of those
+// up to 1 %, and dropping the global tables from theirs up to 5 % ([6|10] 374 -> 392 us), by the compiler's
+// choice of registers alone.
+template <int NR, bool AREAS>
 __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
   extern __shared__ __align__(16) double sm[];
   const PlanDev& P = a.plan;
@@ -77,10 +81,13 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
   uint32_t* rowE = cdt + Nk;                                    // per one-axis ab: E block start, length
   uint32_t* colE = rowE + nab1;                                 // per one-axis cd
   int* area = reinterpret_cast<int*>(colE + ncd1);              // of the tables in global memory
-  const bool stash = P.ry_stash != 0;
-  if (stash && tid == 0) {
-    *area = a.rys_used ? take_area(a.rys_used, a.rys_areas, (int)(blockIdx.x % (unsigned)a.rys_areas)) : (int)blockIdx.x;
-    if (*area < 0) atomicExch(a.err, kDevTimeout);
+  const bool stash = AREAS || P.ry_stash != 0;
+  double* gtab = stash ? a.rys_tab + (int64_t)blockIdx.x * a.rys_stride : tab;
+  if constexpr (AREAS) {
+    if (tid == 0) {
+      *area = take_area(a.rys_used, a.rys_areas, (int)(blockIdx.x % (unsigned)a.rys_areas));
+      if (*area < 0) atomicExch(a.err, kDevTimeout);
+    }
   }
 
   for (int e = tid; e < Nb; e += T) {
@@ -105,9 +112,11 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
     const int x = e / (ld + 1), y = e - x * (ld + 1);
     colE[e] = (uint32_t)eoff(ld, x, y) | (uint32_t)(x + y + 1) << 16;
   }
-  __syncthreads();
-  if (stash && *area < 0) return;
-  double* gtab = stash ? a.rys_tab + *area * a.rys_stride : tab;
+  if constexpr (AREAS) {
+    __syncthreads();
+    if (*area < 0) return;
+    gtab = a.rys_tab + *area * a.rys_stride;
+  }
   const int EB = (P.recb - kRecHeader) / 3, EK = (P.reck - kRecHeader) / 3;   // one axis of a record's tables
   // (the record is padded to an even length: the table length is the integer part)
 
@@ -227,7 +236,7 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
       }
     }
   }
-  if (stash && a.rys_used) {
+  if constexpr (AREAS) {
     __syncthreads();   // every thread has read its tables
     if (tid == 0) {
       __threadfence();
@@ -238,22 +247,23 @@ __global__ void __launch_bounds__(512) k_rys(const QuartetLaunch a) {
 
 using RysKernel = void (*)(const QuartetLaunch);
 template <int... I>
-RysKernel rys_kernel(int n, std::integer_sequence<int, I...>) {
-  static const RysKernel table[] = {k_rys<I + 1>...};
-  return table[n - 1];
+RysKernel rys_kernel(int n, bool areas, std::integer_sequence<int, I...>) {
+  static const RysKernel table[2][kRysMax] = {{k_rys<I + 1, false>...}, {k_rys<I + 1, true>...}};
+  return table[areas][n - 1];
 }
-RysKernel rys_kernel(int n) {
-  return n >= 1 && n <= kRysMax ? rys_kernel(n, std::make_integer_sequence<int, kRysMax>{}) : nullptr;
+RysKernel rys_kernel(int n, bool areas) {
+  return n >= 1 && n <= kRysMax ? rys_kernel(n, areas, std::make_integer_sequence<int, kRysMax>{}) : nullptr;
 }
 
 }  // namespace
 
 cudaError_t rys_attributes_init() {
-  for (int n = 1; n <= kRysMax; ++n) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(rys_kernel(n), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
-  }
+  for (int n = 1; n <= kRysMax; ++n)
+    for (const bool areas : {false, true}) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(rys_kernel(n, areas), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      if (e != cudaSuccess) return e;
+    }
   return cudaSuccess;
 }
 
@@ -263,13 +273,19 @@ cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid, int* resident) {
     *grid = (int)std::min<int64_t>(nq, 0x7fffffff);
     return cudaSuccess;
   }
-  int bps = 0, dev = 0, sms = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, rys_kernel(P.rys), P.ry_threads,
-                                                                (size_t)P.ry_doubles * sizeof(double));
+  int bps = 1, dev = 0, sms = 0;   // blocks per SM: the larger number of the two instances
+  cudaError_t e = cudaSuccess;
+  for (const bool areas : {false, true}) {
+    int n = 0;
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rys_kernel(P.rys, areas), P.ry_threads,
+                                                        (size_t)P.ry_doubles * sizeof(double));
+    bps = std::max(bps, n);
+  }
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  *resident = std::max(1, bps) * sms;
+  *resident = bps * sms;
   *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nq, *resident));
   return cudaSuccess;
 }
@@ -277,7 +293,7 @@ cudaError_t rys_grid(const PlanDev& P, int64_t nq, int* grid, int* resident) {
 cudaError_t launch_rys(const QuartetLaunch& a, int grid, cudaStream_t s) {
   if (a.nq <= 0) return cudaSuccess;
   const PlanDev& P = a.plan;
-  const RysKernel k = rys_kernel(P.rys);
+  const RysKernel k = rys_kernel(P.rys, P.ry_stash && a.rys_used);
   if (!k || !a.rys || a.D || a.grad || grid < 1) return cudaErrorInvalidValue;
   if (P.ry_stash && (!a.rys_tab || a.rys_stride < P.ry_table || a.rys_areas < (a.rys_used ? 1 : grid)))
     return cudaErrorInvalidValue;
