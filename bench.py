@@ -41,8 +41,8 @@ UNIT = "GFLOP/s (Table-1 model FLOPs)"
 FP64_FLOP_PER_CLK_SM = 4.0
 CHUNK_BYTES = 2 << 30
 # DRAM bytes (read + write) per [ii|ii] quartet of one k_rys launch of the benchmark (456 quartets), from the
-# capture whose command is in profiles/k_rys_ii_bench_launch.md: 1,000,510,464 B read + 2,647,006,464 B written
-NCU_DRAM_BYTES_PER_II_QUARTET = (1000510464 + 2647006464) / 456
+# capture whose command is in profiles/k_rys_ii_bench_launch.md: 1,005,679,616 B read + 2,649,168,640 B written
+NCU_DRAM_BYTES_PER_II_QUARTET = (1005679616 + 2649168640) / 456
 
 
 def parse():

@@ -173,7 +173,14 @@ mdx_status mdx_eri3_sph(mdx_ctx* ctx, const mdx_basis* aux, const mdx_basis* orb
  * destroyed; the batch keeps its own copies of the index data. The per-class
  * launches of a run are spread over the caller's stream and the context's
  * internal streams, ordered after the work already queued on the caller's
- * stream, which waits for all of them. */
+ * stream, which waits for all of them.
+ * Uncontracted Cartesian classes without a register kernel run the Rys kernel:
+ * the first of a process builds its node table on the host (0.1 s on eight
+ * cores, 0.9 s on one), and each context uploads it once (1.9 MB). Classes
+ * above [gg|gg] keep axis tables in device memory that the context's prepared
+ * batches share (114 MB for [ii|ii], up to 228 MB; freed with the last of
+ * them; MDX_ENOMEM if it cannot be had); one-shot calls keep theirs in
+ * context workspace. */
 typedef struct mdx_batch mdx_batch;
 
 /* Prepare the quartets of mdx_eri4 (same arguments, without screening
