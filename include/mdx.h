@@ -178,9 +178,9 @@ mdx_status mdx_eri3_sph(mdx_ctx* ctx, const mdx_basis* aux, const mdx_basis* orb
  * the first of a process builds its node table on the host (0.1 s on eight
  * cores, 0.9 s on one), and each context uploads it once (1.9 MB). Classes
  * above [gg|gg] keep axis tables in device memory that the context's prepared
- * batches share (114 MB for [ii|ii], up to 228 MB; freed with the last of
- * them; MDX_ENOMEM if it cannot be had); one-shot calls keep theirs in
- * context workspace. */
+ * batches share and the context keeps (114 MB for [ii|ii], up to 228 MB;
+ * MDX_ENOMEM if it cannot be had); one-shot calls keep theirs in context
+ * workspace. */
 typedef struct mdx_batch mdx_batch;
 
 /* Prepare the quartets of mdx_eri4 (same arguments, without screening

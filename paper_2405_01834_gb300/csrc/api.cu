@@ -39,16 +39,14 @@ struct NvtxRange {
 
 // Axis tables of the Rys classes that keep them in global memory: `areas` of `stride` doubles, as many as their blocks
 // that the GPU holds at a time, each taken by a block while it runs (`used`). The prepared batches of a context
-// share one (114 MB for [ii|ii]); it goes with the last batch that uses it.
+// share one (114 MB for [ii|ii]), which the context keeps: the preparation of a batch of 441 [ii|ii] quartets takes 290 us
+// where it allocates an area, 210 where it finds one. One that a larger one has replaced goes with the last batch that uses it.
 struct RysAreas {
   double* tab = nullptr;
-  int32_t* used = nullptr;
+  int32_t* used = nullptr;   // behind the tables, in the same allocation
   int64_t stride = 0;
   int areas = 0;
-  ~RysAreas() {
-    cudaFree(tab);
-    cudaFree(used);
-  }
+  ~RysAreas() { cudaFree(tab); }
 };
 
 struct mdx_ctx {
@@ -56,7 +54,7 @@ struct mdx_ctx {
   std::string last_error;
   double* d_boys = nullptr;
   double* d_rys = nullptr;                // Rys nodes and weights, uploaded when a class first needs them
-  std::weak_ptr<RysAreas> rys_areas;      // the batches' newest areas
+  std::shared_ptr<RysAreas> rys_areas;    // of the prepared batches
   uint32_t* d_rprog = nullptr;
   int32_t* d_rprog_off = nullptr;
   int* d_err = nullptr;
@@ -191,9 +189,10 @@ mdx_status need_rys_table(mdx_ctx* c, cudaStream_t s) {
   return MDX_OK;
 }
 
-// Areas of at least `stride` doubles, at least `n` of them: the batches' present ones, or new ones that serve both.
+// Areas of at least `stride` doubles, at least `n` of them: the batches' present ones, or new ones that serve both. Runs on
+// other streams come after the zeroing on `s`, for which the preparation of the batch waits.
 mdx_status need_rys_areas(mdx_ctx* c, int64_t stride, int n, std::shared_ptr<RysAreas>* out, cudaStream_t s) {
-  const std::shared_ptr<RysAreas> cur = c->rys_areas.lock();
+  const std::shared_ptr<RysAreas> cur = c->rys_areas;
   if (cur && cur->stride >= stride && cur->areas >= n) {
     *out = cur;
     return MDX_OK;
@@ -201,13 +200,13 @@ mdx_status need_rys_areas(mdx_ctx* c, int64_t stride, int n, std::shared_ptr<Rys
   auto a = std::make_shared<RysAreas>();
   a->stride = cur ? std::max(stride, cur->stride) : stride;
   a->areas = cur ? std::max(n, cur->areas) : n;
-  if (cudaMalloc(&a->tab, (size_t)a->areas * a->stride * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&a->used, (size_t)a->areas * sizeof(int32_t)) != cudaSuccess) {
+  const size_t doubles = (size_t)a->areas * a->stride, words = (size_t)a->areas * sizeof(int32_t);
+  if (cudaMalloc(&a->tab, doubles * sizeof(double) + words) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, MDX_ENOMEM, "Rys table area allocation failed");
   }
-  cudaError_t e = cudaMemsetAsync(a->used, 0, (size_t)a->areas * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // runs on other streams come after it
+  a->used = (int32_t*)(a->tab + doubles);
+  const cudaError_t e = cudaMemsetAsync(a->used, 0, words, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "Rys table area");
   c->rys_areas = a;
   *out = a;

@@ -74,18 +74,20 @@ def test_captured_runs_replayed_side_by_side():
 
 
 def test_areas_are_shared_and_given_back():
-    """The batches of an engine share one set of areas (152 x 749 KB for [ii|ii]); it goes with the last of them."""
+    """The batches of an engine share one set of areas (152 x 749 KB for [ii|ii]), whichever of them is closed, and the
+    engine gives it back."""
     eng = mdx.Engine(0)
     b, q = inputs.class_sweep((6, 6, 6, 6), n_bra=1, n_ket=1, seed=31)
     db = mdx.DeviceBasis(b)
     free = lambda: torch.cuda.mem_get_info()[0]  # noqa: E731
-    eng.batch_eri4(db, q).close()   # plans and node table, which stay
+    area = 152 * 749112
     torch.cuda.synchronize()
     before = free()
     first = eng.batch_eri4(db, q)
     used = before - free()
+    assert used >= area
     more = [eng.batch_eri4(db, q) for _ in range(8)]
-    assert before - free() < used + used // 2
+    assert before - free() < used + area // 2
     first.close()
     o = _out(more[0])
     more[0].run(o)
@@ -93,5 +95,8 @@ def test_areas_are_shared_and_given_back():
     assert torch.isfinite(o).all()
     for x in more:
         x.close()
-    assert before - free() < used // 2
+    B = eng.batch_eri4(db, q)
+    assert before - free() < used + area // 2
+    B.close()
     eng.close()
+    assert before - free() < area // 2
