@@ -1,5 +1,4 @@
 """Runs of prepared batches that overlap on the GPU: the Rys classes whose axis tables live in global memory."""
-import numpy as np
 import pytest
 import torch
 

@@ -1,5 +1,4 @@
 """The shares of small launches (lanes and teams per quartet) depend on the call alone."""
-import numpy as np
 import pytest
 import torch
 
